@@ -173,3 +173,45 @@ def run(s):
         s["graph"].replay()
         return s["outs"]
     return bd.gemm(s["X"], s["W"], s["bits"], s["alpha"], out=s["out"], workspace=s["ws"], bias=s["bias"], act=s["act"])
+
+
+def _signs64(bits, b):
+    """+1 / -1 of tenant b as [N, K] in 64 bits."""
+    j = torch.arange(32, device="cuda", dtype=torch.int32)
+    return (((bits[b].unsqueeze(-1) >> j) & 1).to(torch.float64) * 2 - 1).reshape(bits.shape[1], -1)
+
+
+def _product64(X, W, bits, alpha, bias, act):
+    base = W.double()
+    Y = []
+    for b in range(X.shape[0]):
+        x = X[b].double()
+        z = x @ base.t() + alpha[b].double() * (x @ _signs64(bits, b).t())
+        if bias is not None:
+            z = z + bias.double()
+        if act == "silu":
+            z = z * torch.sigmoid(z)
+        elif act == "silu_gate":
+            z = z[:, 0::2] * torch.sigmoid(z[:, 0::2]) * z[:, 1::2]
+        Y.append(z)
+    return torch.stack(Y)
+
+
+def exact(case, seed):
+    s = prepare(case, seed)
+    if case["op"] == "compress":
+        base, bits, alpha = s["base"].double(), [], []
+        j = torch.arange(32, device="cuda", dtype=torch.int64)
+        for fine in s["fine"]:
+            delta = fine.double() - base
+            word = ((delta > 0).reshape(case["N"], -1, 32).long() << j).sum(-1)
+            bits.append(torch.where(word >= 2**31, word - 2**32, word).to(torch.int32))
+            alpha.append(delta.abs().mean())
+        return torch.stack(bits), torch.stack(alpha)
+    if case["op"] == "layer":
+        y, outs = s["x"], []
+        for W, bits, alpha, _, _, act in s["parts"]:
+            y = _product64(y, W, bits, alpha, None, act)
+            outs.append(y)
+        return outs
+    return _product64(s["X"], s["W"], s["bits"], s["alpha"], s["bias"], s["act"])
