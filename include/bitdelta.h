@@ -104,7 +104,9 @@ int bitdelta_workspace_init(void* workspace, size_t workspace_bytes, void* cuda_
  * schedule (several tenants per tile up to m = 64; pairs of thread blocks with
  * 256-row MMAs for m > 64); all run on tcgen05 tensor cores with TMEM
  * accumulators, and bitdelta_gemm_plan tells which one a shape gets.  Shapes
- * whose K is not a multiple of 128 run on a plain CUDA-core kernel instead.
+ * whose K is not a multiple of 128 take the tiled schedule for every m, or a plain
+ * CUDA-core kernel: with K < 128, one token against a small matrix, or without
+ * the workspace that the tiled schedule needs.
  * X, W_base, bits and Y must be 16-byte aligned; K a multiple of 32.
  * Asynchronous on the stream; a kernel-side wait that expires is reported by
  * bitdelta_last_device_status, not here.
@@ -231,7 +233,7 @@ int bitdelta_gemm_host(const void* X_host, const void* W_base_host, const uint32
  *
  * bitdelta_gemm_plan fills info[0 .. BITDELTA_PLAN_INFO_INTS-1] (host pointer):
  *   [0] schedule: 0 tiled, 1 decode with a pre-pass activation split, 2 decode with the in-kernel split,
- *       3 CUDA-core kernel (K not a multiple of 128; all other entries are 0 then), 4 tiled on pairs of
+ *       3 CUDA-core kernel (K not a multiple of 128 and a small product; all other entries are 0 then), 4 tiled on pairs of
  *       thread blocks (a unit is then two W_base tiles, [3] and the work list count such pairs, and [1] is
  *       twice the number of pairs that cut the list), 7 / 8 the 4-bit decode kernel on
  *       the flat work list / in clusters (8 is the default wherever it applies: m <= 8, one tenant group,

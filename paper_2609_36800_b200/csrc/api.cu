@@ -105,11 +105,25 @@ int check_gemm_args(const void* X, const void* W, const void* bits, const void* 
 bool encode_bf16_tile(CUtensorMap* map, const void* ptr, uint64_t rows, uint64_t K, uint32_t box_rows) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
-    cuuint64_t dims[3] = {64, rows, K / 64};
+    cuuint64_t dims[3] = {64, rows, K / 128 * 2};   // (whole 128-k steps)
     cuuint64_t strides[2] = {K * 2, 128};
     cuuint32_t box[3] = {64, box_rows, 2};
     cuuint32_t estr[3] = {1, 1, 1};
     return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// The last K % 128 columns of a bf16 [rows, K] matrix (`ptr`: their first one), box = one 64-column atom x box_rows;
+// columns past the matrix are zero-filled.  (x = 0 or 64: 128-byte aligned.)
+bool encode_bf16_tail(CUtensorMap* map, const void* ptr, uint64_t rows, uint64_t K, uint32_t box_rows) {
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return false;
+    cuuint64_t dims[2] = {K % 128, rows};
+    cuuint64_t strides[1] = {K * 2};
+    cuuint32_t box[2] = {64, box_rows};
+    cuuint32_t estr[2] = {1, 1};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -269,8 +283,8 @@ int bitdelta_compress(const void* W_fine, const void* W_base, uint32_t* bits, fl
 
 size_t bitdelta_gemm_workspace_bytes(int B, int m, int N, int K) {
     if (B <= 0 || m <= 0 || N <= 0 || K <= 0 || (K % 32) != 0) return 0;
-    if ((K % 128) != 0) return 256;   // CUDA-core path: no scratch needed, keep the pointer non-NULL
     bd::Plan p = bd::make_plan(B, m, N, K, 148, tb_override(), whole_override());
+    if ((K % 128) != 0 && !p.ok) return 256;   // CUDA-core path: no scratch needed, keep the pointer non-NULL
     if (!p.ok) return 0;
     size_t need = p.ws_bytes;
     if (p.decode) {   // the same shape on the tiled schedule (BITDELTA_DTYPE_WIDE_RANGE) may need more
@@ -328,14 +342,6 @@ int bitdelta_gemm_ex(const void* X, const void* W_base, const uint32_t* bits, co
     if (st != BITDELTA_OK) return st;
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
 
-    if ((K % 128) != 0) {
-        // Row pitch of the sign words is not a multiple of 16 bytes: no tensor map exists for it.
-        if (bd::launch_gemm_simt(X, W_base, bits, alpha, bias, Y, B, m, N, K, f16, act, stream) != cudaSuccess)
-            return BITDELTA_ERR_CUDA;
-        g_launches++;
-        return BITDELTA_OK;
-    }
-
     const bool plain = !f16 && act == BITDELTA_ACT_NONE && bias == nullptr;   // (the 4-bit decode kernel takes no options)
     bd::Plan p = bd::make_plan(B, m, N, K, d.sms, tb_override(), whole_override(), true, wide, plain);
     if (p.ok && p.pair) {
@@ -371,6 +377,14 @@ int bitdelta_gemm_ex(const void* X, const void* W_base, const uint32_t* bits, co
         const int need = p.grid / p.cluster;
         if (n < need) p = bd::make_plan(B, m, N, K, d.sms, tb_override(), whole_override(), false, false, plain);
     }
+    if ((K % 128) != 0 && (!p.ok || !workspace || workspace_bytes < p.ws_bytes || !aligned16(workspace))) {
+        // K < 128, a work list beyond the split arithmetic, or no scratch for the tiled schedule (the no-allocation
+        // entry point with a large shape): the CUDA-core kernel, which needs none.
+        if (bd::launch_gemm_simt(X, W_base, bits, alpha, bias, Y, B, m, N, K, f16, act, stream) != cudaSuccess)
+            return BITDELTA_ERR_CUDA;
+        g_launches++;
+        return BITDELTA_OK;
+    }
     if (!p.ok) return BITDELTA_ERR_SHAPE;
     if (!workspace || workspace_bytes < p.ws_bytes) return BITDELTA_ERR_WORKSPACE;
     if (!aligned16(workspace)) return BITDELTA_ERR_ALIGN;
@@ -383,10 +397,20 @@ int bitdelta_gemm_ex(const void* X, const void* W_base, const uint32_t* bits, co
                                  [&](CUtensorMap* mp) { return encode_bf16_tile(mp, X, (uint64_t)B * m, (uint64_t)K, (uint32_t)p.x_rows); }))
         return BITDELTA_ERR_CUDA;
     const uint32_t box_words = (p.fp4 && p.bits_row == 16) ? 4u : 8u;
-    if (!cached_map(&tmBits, MapKey{1, bits, (uint64_t)B, (uint64_t)N, (uint64_t)(K / 32), (uint32_t)p.TB, box_words},
+    if (!p.ragged && !cached_map(&tmBits, MapKey{1, bits, (uint64_t)B, (uint64_t)N, (uint64_t)(K / 32), (uint32_t)p.TB, box_words},
                     [&](CUtensorMap* mp) { return encode_bits_3d(mp, bits, (uint64_t)B, (uint64_t)N, (uint64_t)(K / 32), (uint32_t)p.TB, box_words); }))
         return BITDELTA_ERR_CUDA;
-    if (p.fp4) {
+    if (p.ragged) {
+        // the short last k-step of W_base and of the activations
+        const uint64_t k_full = (uint64_t)(K / bd::kPairK * bd::kPairK);
+        const uint16_t* Wt = static_cast<const uint16_t*>(W_base) + k_full;
+        const uint16_t* Xt = static_cast<const uint16_t*>(X) + k_full;
+        if (!cached_map(&tmX8, MapKey{3, Wt, (uint64_t)N, (uint64_t)K, 0, (uint32_t)bd::kTileN, 0u},
+                        [&](CUtensorMap* mp) { return encode_bf16_tail(mp, Wt, (uint64_t)N, (uint64_t)K, bd::kTileN); }) ||
+            !cached_map(&tmBits, MapKey{3, Xt, (uint64_t)B * m, (uint64_t)K, 0, (uint32_t)p.x_rows, 0u},
+                        [&](CUtensorMap* mp) { return encode_bf16_tail(mp, Xt, (uint64_t)B * m, (uint64_t)K, (uint32_t)p.x_rows); }))
+            return BITDELTA_ERR_CUDA;
+    } else if (p.fp4) {
         // 4-bit decode kernel: the activation operands of every (tenant group, 128-k step) as shared-memory images, and
         // the token rows' fixed-point units; then the GEMM, which prefetches weights while this is still running.
         uint8_t* img = bd::ws_x8(p, workspace);
@@ -411,7 +435,7 @@ int bitdelta_gemm_ex(const void* X, const void* W_base, const uint32_t* bits, co
 
     bd::GemmArgs args = bd::make_args(p, alpha, Y, workspace);
     args.f16 = f16; args.act = act; args.bias = bias;
-    args.X = X;
+    args.X = X; args.bits = bits;
     { static int h = -1; if (h < 0) { const char* e = getenv("BITDELTA_HOLD"); h = (e && e[0] == '0') ? 0 : 1; } args.hold_prefetch = h; }
     // (a GEMM queued right behind the library's own pack / compress must not prefetch what they are still writing)
     const bool early = early_start_enabled() && g_weights_just_written.exchange(0) == 0;
@@ -479,8 +503,8 @@ int bitdelta_gemm_plan(int B, int m, int N, int K, int num_sms, int* info) {
     if (!info) return BITDELTA_ERR_NULL;
     if (B <= 0 || m <= 0 || N <= 0 || K <= 0 || (K % 32) != 0 || num_sms <= 0) return BITDELTA_ERR_SHAPE;
     for (int i = 0; i < BITDELTA_PLAN_INFO_INTS; ++i) info[i] = 0;
-    if ((K % 128) != 0) { info[0] = 3; return BITDELTA_OK; }
     bd::Plan p = bd::make_plan(B, m, N, K, num_sms, tb_override(), whole_override());
+    if ((K % 128) != 0 && !p.ok) { info[0] = 3; return BITDELTA_OK; }
     if (!p.ok) return BITDELTA_ERR_SHAPE;
     info[0] = !p.decode ? (p.pair ? 4 : 0) : p.fp4 ? (p.cluster > 1 ? 8 : 7) : (p.convert ? 2 : 1);
     info[1] = p.grid; info[2] = p.TB; info[3] = p.units; info[4] = p.P;
@@ -556,7 +580,8 @@ int bitdelta_gemm_noalloc(const void* X, const void* W_base, const uint32_t* bit
     if (st != BITDELTA_OK) return st;
     const size_t need = bitdelta_gemm_workspace_bytes(B, m, N, K);
     if (need == 0) return BITDELTA_ERR_SHAPE;
-    if (need > (size_t)BITDELTA_NOALLOC_SCRATCH_BYTES) return BITDELTA_ERR_WORKSPACE;
+    if (need > (size_t)BITDELTA_NOALLOC_SCRATCH_BYTES && (K % 128) == 0)   // (other K: the CUDA-core kernel needs no scratch)
+        return BITDELTA_ERR_WORKSPACE;
 
     // Device address of the scratch array, looked up once per device with that device current.
     static void* scratch_ptr[64] = {};
@@ -574,9 +599,9 @@ int bitdelta_gemm_noalloc(const void* X, const void* W_base, const uint32_t* bit
     }
     // The arrival counters at the start of the scratch have to be zero when the kernel begins; a call
     // that was cut short could have left them otherwise.
-    if ((K % 128) == 0) {
-        bd::Plan plan = bd::make_plan(B, m, N, K, d.sms, tb_override(), whole_override());
-        if (!plan.ok) return BITDELTA_ERR_SHAPE;
+    bd::Plan plan = bd::make_plan(B, m, N, K, d.sms, tb_override(), whole_override());
+    if (!plan.ok && (K % 128) == 0) return BITDELTA_ERR_SHAPE;
+    if (plan.ok && plan.ws_bytes <= (size_t)BITDELTA_NOALLOC_SCRATCH_BYTES) {
         if (cudaMemsetAsync(scratch, 0, plan.ws_header_bytes, static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess)
             return BITDELTA_ERR_CUDA;
     }

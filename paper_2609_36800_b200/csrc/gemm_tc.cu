@@ -37,6 +37,7 @@ constexpr int kWarpTmem = 2;
 constexpr int kWarpDelta0 = 2;     // decode schedule: warps 2..3 issue the delta MMAs of decode group 0 / 1
 constexpr int kBarAFull0 = 2;      // named barriers 2..9 : decode group g, buffer b -> id 2 + g*4 + b
 constexpr int kWarpDecode0 = 4;    // warps 4..11
+constexpr int kRaggedBitThreads = 64;   // tiled schedule, K % 128 != 0: warps 2..3 copy the sign words
 constexpr int kWarpEpi0 = 12;      // warps 12..15
 
 struct Ctl {
@@ -66,7 +67,8 @@ static_assert(sizeof(Ctl) <= kSmemCtrlBytes, "control block too large");
 // instruction caches) and turns the schedule switches into compile-time constants.
 // kGen: the general form (binary16 I/O, bias, activation); false compiles the plain bf16 product alone, whose
 // code is then exactly as short as it can be (the kernel's speed is sensitive to its length).
-template <int kMode, bool kGen>
+// kRagged: K % 128 != 0 (tiled modes, general form); a form of its own because the run-time test cost the others 2 %.
+template <int kMode, bool kGen, bool kRagged = false>
 __global__ void __launch_bounds__(kThreads, 1)
 bitdelta_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX,
                         const __grid_constant__ CUtensorMap tmX8, const __grid_constant__ CUtensorMap tmBits,
@@ -96,6 +98,11 @@ bitdelta_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
     const int am = ((kMode >= 1 && kMode <= 4) || kMode == 8) ? kMode : a.m;
     const bool convert = kDec && a.convert != 0;
     const bool io_f16 = kGen && a.f16 != 0;
+    // K % 128 != 0: the weights' and activations' last, short k-step is loaded through
+    // tensor maps of its own whose extent ends with the row (the rest of the tile is zero-filled): tmX8 holds W_base's,
+    // tmBits the activations'.
+    constexpr bool ragged = kRagged;
+    static_assert(!kRagged || (kGen && !kDec), "the ragged form is built for the tiled schedules' general form");
     auto unit_info = [&](const GemmArgs& aa, int un) { return unit_info_t<kDec, kGrouped, kPair>(aa, un, am, (int)rank); };
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
@@ -128,14 +135,25 @@ bitdelta_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
             // Both CTAs' tiles of the stage (W_base and half an activation tile each) are counted on the
             // leader's barrier, which only the leader arms.
             if (rank == 0) mbar_arrive_expect_tx(bar, 2u * (a.w_stage_bytes + 2 * a.x_atom_bytes));
-            tma_load_3d_pair(dst, &tmW, mapa_shared(bar, 0), 0, u.n0, k0 / kAtomK);
+            const uint32_t lbar = mapa_shared(bar, 0);
+            if (ragged && p == a.P - 1) {
+                tma_load_2d_pair(dst, &tmX8, lbar, 0, u.n0);
+                tma_load_2d_pair(dst + a.w_atom_bytes, &tmX8, lbar, kAtomK, u.n0);
+            } else {
+                tma_load_3d_pair(dst, &tmW, lbar, 0, u.n0, k0 / kAtomK);
+            }
         } else {
             // tiled schedule: the stage's activation tile (same slot index, queued by the activation
             // stream) completes on this barrier too
             mbar_arrive_expect_tx(bar, a.w_stage_bytes + (kDec ? 0u : 2 * a.x_atom_bytes));
-            tma_load_3d(dst, &tmW, bar, 0, u.n0, k0 / kAtomK);   // both 64-k atoms of the tile
+            if (ragged && p == a.P - 1) {
+                tma_load_2d(dst, &tmX8, bar, 0, u.n0);
+                tma_load_2d(dst + a.w_atom_bytes, &tmX8, bar, kAtomK, u.n0);
+            } else {
+                tma_load_3d(dst, &tmW, bar, 0, u.n0, k0 / kAtomK);   // both 64-k atoms of the tile
+            }
         }
-        if (with_bits) {
+        if (with_bits && !ragged) {
             const uint32_t bbar = smem_u32(&ctl->bfull[bslot]);
             mbar_arrive_expect_tx(bbar, a.bslot_bytes);
             tma_load_3d(bits_addr + bslot * a.bslot_bytes, &tmBits, bbar, (p >> 1) * 8, u.n0, u.tenant0);
@@ -164,7 +182,7 @@ bitdelta_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
             mbar_init(smem_u32(&ctl->x8empty[s]), 2);                            // the two delta issuers
         }
         for (int s = 0; s < kMaxBitSlots; ++s) {
-            mbar_init(smem_u32(&ctl->bfull[s]), 1);
+            mbar_init(smem_u32(&ctl->bfull[s]), ragged ? kRaggedBitThreads : 1);   // (ragged: every copying thread)
             mbar_init(smem_u32(&ctl->bempty[s]), kDec ? 8 : 4);
         }
         for (int s = 0; s < kMaxASlots; ++s) mbar_init(smem_u32(&ctl->afull[s]), kPair ? 8 : 4);   // (pair: both CTAs' decode warps)
@@ -237,7 +255,7 @@ bitdelta_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
         // deep ring), so that they run far ahead of the W_base tiles: the decode warps work several stages
         // ahead of the MMAs.  In the decode schedules they travel with the W_base stream.
         ItemIter bi(it);
-        bool more_b = !kDec && bi.next();
+        bool more_b = !kDec && !ragged && bi.next();
         Unit ub{};
         auto next_pair = [&]() {   // to the next item that starts a k-pair of its segment
             do {
@@ -272,10 +290,22 @@ bitdelta_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
                         const int k0 = xi.p * kPairK;
                         if constexpr (kPair) {
                             // this CTA's half of the token tile, counted on the leader's barrier
-                            tma_load_3d_pair(dst, &tmX, mapa_shared(bar, 0), 0, ux.xrow0 + (int)rank * (a.tok_tile / 2), k0 / kAtomK);
+                            const uint32_t lbar = mapa_shared(bar, 0);
+                            const int xrow = ux.xrow0 + (int)rank * (a.tok_tile / 2);
+                            if (ragged && xi.p == a.P - 1) {
+                                tma_load_2d_pair(dst, &tmBits, lbar, 0, xrow);
+                                tma_load_2d_pair(dst + a.x_atom_bytes, &tmBits, lbar, kAtomK, xrow);
+                            } else {
+                                tma_load_3d_pair(dst, &tmX, lbar, 0, xrow, k0 / kAtomK);
+                            }
                         } else {
                             if (kDec) mbar_arrive_expect_tx(bar, a.x_tile_bytes);
-                            tma_load_3d(dst, &tmX, bar, 0, ux.xrow0, k0 / kAtomK);   // both 64-k atoms
+                            if (ragged && xi.p == a.P - 1) {
+                                tma_load_2d(dst, &tmBits, bar, 0, ux.xrow0);
+                                tma_load_2d(dst + a.x_atom_bytes, &tmBits, bar, kAtomK, ux.xrow0);
+                            } else {
+                                tma_load_3d(dst, &tmX, bar, 0, ux.xrow0, k0 / kAtomK);   // both 64-k atoms
+                            }
                         }
                     }
                     __syncwarp();
@@ -533,6 +563,37 @@ bitdelta_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
                 __syncwarp();
                 accphase ^= 1;
             }
+        } else if (ragged) {
+            // ------------------------------------------- sign words (tiled schedule, K % 128 != 0)
+            // The row pitch of the sign words is a multiple of 4 bytes only, so no tensor map takes them: these two
+            // otherwise idle warps copy them word by word into the slots (eight consecutive lanes take the eight words
+            // of a row: 32 contiguous bytes), as far ahead as the ring allows.  Words past the row's end and
+            // rows past N are zero-filled; the zero-filled activations of the short step make them count for nothing.
+            const int btid = (int)threadIdx.x - kWarpDelta0 * 32;
+            const int words = a.K >> 5;
+            ItemIter bi(it);
+            int bslot = 0;
+            uint32_t bphase = 0;
+            bool ok = true;
+            while (ok && bi.next()) {
+                if (!bi.first && (bi.p & 1)) continue;   // (in the slot of the step before it)
+                const Unit u = unit_info(a, bi.unit);
+                ok = warp_all(wait_bar(smem_u32(&ctl->bempty[bslot]), bphase ^ 1, abort_flag, 16));
+                if (!ok) break;
+                const int wd = (bi.p >> 1) * 8 + (btid & 7);
+                for (int j = 0; j < u.nten; ++j) {
+                    const uint32_t dst = bits_addr + bslot * a.bslot_bytes + (uint32_t)(j * kTileN * 32 + btid * 4);
+                    const uint32_t* src = a.bits + ((size_t)(u.tenant0 + j) * a.N + u.n0 + (btid >> 3)) * words + wd;
+#pragma unroll 4
+                    for (int r = 0; r < kTileN; r += kRaggedBitThreads / 8) {
+                        const bool in = wd < words && u.n0 + (btid >> 3) + r < a.N;
+                        cp_async_4(dst + (uint32_t)r * 32, in ? src + (size_t)r * words : a.bits, in ? 4u : 0u);
+                    }
+                }
+                cp_async_mbar_arrive(smem_u32(&ctl->bfull[bslot]));
+                if (++bslot == a.n_bits) { bslot = 0; bphase ^= 1; }
+            }
+            cp_async_wait_all();
         }
     } else if (warp >= kWarpDecode0 && warp < epi_first_warp) {
         // ------------------------------------------- sign decode -> tensor memory
@@ -925,17 +986,19 @@ cudaError_t launch_gemm_tc(const CUtensorMap& tmW, const CUtensorMap& tmX, const
     const int gen = (args.f16 || args.act || args.bias != nullptr) ? 9 : 0;
     // 0 tiled, 1..4 and 8 decode with that many tokens per tenant, 5 decode with any other number up to 16, 6 tiled with
     // several tenants per unit, 7 tiled on CTA pairs
-    const int mode = gen + (!args.decode ? (args.pair ? 7 : (args.win_rows > 0 ? 6 : 0)) : (args.m <= 4 ? args.m : (args.m == 8 ? 8 : 5)));
+    // (18 .. 20: tiled, several tenants, pairs with K % 128 != 0, general form)
+    const int mode = args.ragged ? (args.pair ? 20 : (args.win_rows > 0 ? 19 : 18)) : gen + (!args.decode ? (args.pair ? 7 : (args.win_rows > 0 ? 6 : 0)) : (args.m <= 4 ? args.m : (args.m == 8 ? 8 : 5)));
     using KernelFn = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const GemmArgs);
-    static const KernelFn kernels[18] = {
+    static const KernelFn kernels[21] = {
         bitdelta_gemm_tc_kernel<0, false>, bitdelta_gemm_tc_kernel<1, false>, bitdelta_gemm_tc_kernel<2, false>,
         bitdelta_gemm_tc_kernel<3, false>, bitdelta_gemm_tc_kernel<4, false>, bitdelta_gemm_tc_kernel<5, false>,
         bitdelta_gemm_tc_kernel<6, false>, bitdelta_gemm_tc_kernel<7, false>, bitdelta_gemm_tc_kernel<8, false>,
         bitdelta_gemm_tc_kernel<0, true>,  bitdelta_gemm_tc_kernel<1, true>,  bitdelta_gemm_tc_kernel<2, true>,
         bitdelta_gemm_tc_kernel<3, true>,  bitdelta_gemm_tc_kernel<4, true>,  bitdelta_gemm_tc_kernel<5, true>,
-        bitdelta_gemm_tc_kernel<6, true>,  bitdelta_gemm_tc_kernel<7, true>,  bitdelta_gemm_tc_kernel<8, true>};
+        bitdelta_gemm_tc_kernel<6, true>,  bitdelta_gemm_tc_kernel<7, true>,  bitdelta_gemm_tc_kernel<8, true>,
+        bitdelta_gemm_tc_kernel<0, true, true>, bitdelta_gemm_tc_kernel<6, true, true>, bitdelta_gemm_tc_kernel<7, true, true>};
     // (per device and instantiation, once; setting it twice from two threads is harmless)
-    static std::atomic<unsigned char> attr_done[64][18];
+    static std::atomic<unsigned char> attr_done[64][21];
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;

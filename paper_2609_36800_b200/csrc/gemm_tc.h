@@ -13,6 +13,8 @@ struct GemmArgs {
     int B, m, N, K;
     int decode, convert, TB, tok_tile, Nb, Nd, win_rows, chunk_rows, aslot_cols;
     int pair;            // tiled schedule on CTA pairs (see plan.h)
+    int ragged;          // tiled schedule, K % 128 != 0 (see plan.h)
+    const uint32_t* bits;   // ... sign words [B, N, K/32] for plain loads (the other forms use their tensor map)
     int f16;             // 0: X, W_base, bias, Y are bf16; 1: IEEE binary16
     int act;             // fused epilogue: 0 none, 1 SiLU (after the bias)
     const void* bias;    // [N] values of the I/O type added to every output row, or nullptr
@@ -55,7 +57,7 @@ inline GemmArgs make_args(const Plan& p, const float* alpha, void* Y, void* work
     a.decode = p.decode; a.convert = p.convert; a.TB = p.TB; a.tok_tile = p.tok_tile; a.Nb = p.Nb; a.Nd = p.Nd;
     a.win_rows = p.win_rows; a.chunk_rows = p.chunk_rows; a.aslot_cols = p.aslot_cols;
     a.m_tiles = p.m_tiles; a.groups = p.groups; a.P = p.P; a.T = (int)p.T; a.whole_units = p.whole_units;
-    a.pair = p.pair;
+    a.pair = p.pair; a.ragged = p.ragged;
     a.teams = p.teams; a.Tg = (int)(p.T / p.teams); a.cpt = (p.pair ? p.grid / 2 : p.grid) / p.teams; a.n_tiles = p.n_tiles;
     a.q = a.Tg / a.cpt; a.r = a.Tg % a.cpt;
     a.n_w = p.n_w; a.n_x = p.n_x; a.n_x8 = p.n_x8; a.n_bits = p.n_bits; a.a_slots = p.a_slots; a.hold_prefetch = 1; a.halves = p.halves;

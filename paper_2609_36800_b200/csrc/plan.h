@@ -45,6 +45,8 @@ struct Plan {
                        // tenants x 64 k of e5m2; a_slots buffers per group), tiled 64 (one tenant x 128 k of bf16)
     int n_tiles, m_tiles, groups, units;
     int P;             // k-pairs per unit
+    int ragged;        // tiled schedule, K a multiple of 32 but not of 128: the last k-step is short (zero-filled), the
+                       // sign words (row pitch not a multiple of 16 bytes) come through the load/store unit
     int whole_units;   // 1: CTAs take whole units round-robin (no tile is cut), 0: even shares of the item list
     int teams;         // > 1: one team of grid/teams CTAs per tenant group; units are numbered group-major and each
                        // team cuts its group's items evenly (1: one cut of the whole list, units tile-major)
@@ -124,7 +126,16 @@ inline Plan make_plan(int B, int m, int N, int K, int num_sms, int tb_override =
     Plan p{};
     p.B = B; p.m = m; p.N = N; p.K = K;
     p.ok = false;
-    if (B <= 0 || m <= 0 || N <= 0 || K <= 0 || (K % 128) != 0) return p;
+    if (B <= 0 || m <= 0 || N <= 0 || K <= 0 || (K % 32) != 0) return p;
+    if ((K % kPairK) != 0) {
+        // The tiled schedule for every m: its operands hold both terms in the I/O type, as the CUDA-core kernel does that
+        // such K are otherwise left to (6 x 40 x 2080 x 1999: 3870 -> 21 us).  That kernel keeps the sizes where it is ahead:
+        // less than one whole step, and one token against a small matrix (1 x 1 x 544 x 512: 5.8 us, tiled 6.8; 1 x 1 x 160 x
+        // 4096: 6.6 and 7.4; but 1 x 1 x 4128 x 4096: 73 and 13.8, 1 x 8 x 544 x 512: 23.5 and 7.0).
+        if (K < kPairK || (m == 1 && (long long)B * N * K <= (1ll << 20))) return p;
+        p.ragged = 1;
+        force_tiled = true;
+    }
     p.decode = (m <= kDecodeMaxM && !force_tiled) ? 1 : 0;
     p.n_tiles = (N + kTileN - 1) / kTileN;
     if (p.decode) {
