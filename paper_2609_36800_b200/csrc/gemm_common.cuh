@@ -187,23 +187,46 @@ struct EpiOut {
     int N, n, row, xrow0;
     float bias;         // of output feature n (0 without a bias)
     const GemmArgs& a;  // kernel parameters (activation code, I/O type)
-    // (called by all lanes of a warp together: the gated form exchanges values between neighbouring lanes)
-    __device__ __forceinline__ void put(int tok, float v) const {
+    // Token rows tok .. tok + kTok - 1 of this thread's weight row, the first `nvalid` of them valid (warp-uniform).  The
+    // destination is chosen once per block of tokens and the stores are predicated: with tests and branches per token the
+    // drain of 128 tokens took 6 us, and 3 us even when nothing was stored (two warps per scheduler hide no branch latency).
+    // (Called by all lanes of a warp together: the gated form exchanges values between neighbouring lanes.)
+    template <int kTok>
+    __device__ __forceinline__ void put(int tok, const float (&v)[kTok], int nvalid) const {
         if (slot) {
-            slot[(size_t)tok * kTileN + row] = v;   // partial sums: finished by the CTA that adds them up
+            float* p = slot + (size_t)tok * kTileN + row;   // partial sums: finished by the CTA that adds them up
+#pragma unroll
+            for (int t = 0; t < kTok; ++t)
+                if (t < nvalid) p[t * kTileN] = v[t];
             return;
         }
         if constexpr (kGate) {
             // SiLU gate: weight rows come in pairs (2i: gate, 2i+1: up), i.e. in neighbouring lanes
-            const float z = v + bias;
-            const float other = __shfl_xor_sync(0xFFFFFFFFu, z, 1);
-            if (!(n & 1) && n < N)
-                Y[(size_t)(xrow0 + tok) * (N >> 1) + (n >> 1)] = to_io16(__fdividef(z, 1.f + __expf(-z)) * other, a.f16);
-            return;
-        }
-        if (n < N) {
-            if constexpr (kGen) Y[(size_t)(xrow0 + tok) * N + n] = finish_io16(v, bias, a.act, a.f16);
-            else Y[(size_t)(xrow0 + tok) * N + n] = __bfloat16_as_ushort(__float2bfloat16_rn(v));
+            const int lim = (!(n & 1) && n < N) ? nvalid : 0;
+            uint16_t* p = Y + (size_t)(xrow0 + tok) * (N >> 1) + (n >> 1);
+#pragma unroll
+            for (int t = 0; t < kTok; ++t) {
+                const float z = v[t] + bias;
+                const float other = __shfl_xor_sync(0xFFFFFFFFu, z, 1);
+                const uint16_t o = to_io16(__fdividef(z, 1.f + __expf(-z)) * other, a.f16);
+                if (t < lim) p[(size_t)t * (N >> 1)] = o;
+            }
+        } else {
+            const int lim = n < N ? nvalid : 0;
+            uint16_t* p = Y + (size_t)(xrow0 + tok) * N + n;
+            if (kGen && a.act == 1) {
+#pragma unroll
+                for (int t = 0; t < kTok; ++t) {
+                    const uint16_t o = finish_io16(v[t], bias, 1, a.f16);
+                    if (t < lim) p[(size_t)t * N] = o;
+                }
+            } else {
+#pragma unroll
+                for (int t = 0; t < kTok; ++t) {
+                    const uint16_t o = kGen ? to_io16(v[t] + bias, a.f16) : __bfloat16_as_ushort(__float2bfloat16_rn(v[t]));
+                    if (t < lim) p[(size_t)t * N] = o;
+                }
+            }
         }
     }
 };
@@ -238,12 +261,14 @@ __device__ __forceinline__ void epilogue_decode(const GemmArgs& a, const Unit& u
                 float al;
                 if constexpr (kLoop) al = __shfl_sync(0xFFFFFFFFu, al_lane, j0 + jj);
                 else al = alv[j0 + jj];
+                float v[M];
 #pragma unroll
                 for (int t = 0; t < M; ++t) {
                     const float lo = __uint_as_float(rd[jj * N3 + 2 * M + t]) + __uint_as_float(rd[jj * N3 + 3 * M + t]);
                     const float hi = __uint_as_float(rd[jj * N3 + t]) + __uint_as_float(rd[jj * N3 + M + t]);
-                    out.put((j0 + jj) * M + t, fmaf(al, hi + lo, __uint_as_float(rb[jj * M + t])));
+                    v[t] = fmaf(al, hi + lo, __uint_as_float(rb[jj * M + t]));
                 }
+                out.put((j0 + jj) * M, v, M);
             }
         }
     };
@@ -273,11 +298,10 @@ __device__ __forceinline__ void epilogue_tiled(const GemmArgs& a, const Unit& u,
         tmem_ld32(lane_taddr + a.col_delta + (uint32_t)t0, rd);
         tc_wait_ld();
         if (t0 + 64 >= u.ntok) release();
-        const int nvalid = min(32, u.ntok - t0);
+        float v[32];
 #pragma unroll
-        for (int t = 0; t < 32; ++t) {
-            if (t < nvalid) out.put(t0 + t, fmaf(al, __uint_as_float(rd[t]), __uint_as_float(rb[t])));
-        }
+        for (int t = 0; t < 32; ++t) v[t] = fmaf(al, __uint_as_float(rd[t]), __uint_as_float(rb[t]));
+        out.put(t0, v, u.ntok - t0);
     }
 }
 
@@ -296,18 +320,24 @@ __device__ __forceinline__ void epilogue_tiled_grouped(const GemmArgs& a, const 
         tmem_ld16(lane_taddr + a.col_delta + (uint32_t)(j * a.Nd + t0), rd);
         tc_wait_ld();
         const float al = __shfl_sync(0xFFFFFFFFu, al_lane, j);
-        const int nvalid = min(16, m - t0);
+        float v[16];
 #pragma unroll
-        for (int t = 0; t < 16; ++t) {
-            if (t < nvalid) out.put(j * m + t0 + t, fmaf(al, __uint_as_float(rd[t]), __uint_as_float(rb[t])));
-        }
+        for (int t = 0; t < 16; ++t) v[t] = fmaf(al, __uint_as_float(rd[t]), __uint_as_float(rb[t]));
+        out.put(j * m + t0, v, m - t0);
     }
 }
 
+// Counts one arrival: release of what this thread (and, through a barrier before it, its block) wrote, acquire of the others'.
+__device__ __forceinline__ unsigned atom_add_acq_rel(unsigned int* p) {
+    unsigned old;
+    asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(old) : "l"(p) : "memory");
+    return old;
+}
 __device__ __forceinline__ float4 ldcg4(const float* p) { return __ldcg(reinterpret_cast<const float4*>(p)); }
 
-// Sums the partial results of a tile cut across CTAs c0..c1 (in that order) and writes Y.
-// nwarps*32 threads: thread e owns rows 4*(e%32)..+3 of tokens e/32, e/32+nwarps, ...
+// Sums the partial results of a tile cut across CTAs c0..c1 (in that order) and writes Y.  All warps of the block that
+// arrived last, at the end of its roles: the four or eight epilogue warps alone needed a chain of round trips to L2 (8 us
+// for 80 tokens in three to five parts, now 3).  nwarps*32 threads: thread e owns rows 4*(e%32)..+3 of tokens e/32, e/32+nwarps, ...
 template <bool kGen, bool kGate>
 __device__ __forceinline__ void reduce_partials(const GemmArgs& a, const Unit& u, int etid, int nwarps,
                                                 const float* first, const float* rest, size_t cstride, int nrest) {

@@ -92,7 +92,7 @@ struct FCtl {
     uint64_t tmemready;             // tensor memory is allocated (its base address is in tmem_base)
     uint32_t tmem_base;
     uint32_t abort_flag;
-    uint32_t is_last;
+    uint32_t npend, pend_unit[2];   // cut tiles this block was the last to arrive at: it adds their partials up at the end
     uint64_t imgready[4];           // a step's image is in shared memory and its scale factors in tensor memory (4 epilogue warps)
     uint64_t cntready;              // cooperative image pass: this block has counted itself; img_target is set
     uint32_t img_target;            // ... value of the launch-wide counter at which every block's share is written
@@ -255,13 +255,15 @@ __device__ __forceinline__ void epilogue_fp4(const GemmArgs& a, const Unit& u, u
         if constexpr (ND % 16 >= 8) tmem_ld8(col + ND / 16 * 16, rd + ND / 16 * 16);
         tc_wait_ld();
         const float al = __shfl_sync(0xFFFFFFFFu, al_lane, j) * 6.103515625e-05f;   // tenant j's scale (held by lane j) x 2^-14
+        float v[M];
 #pragma unroll
         for (int t = 0; t < M; ++t) {
             float d = 0.f;
 #pragma unroll
             for (int q = 0; q < kFp4Pieces; ++q) d += __uint_as_float(rd[q * M + t]);
-            out.put(j * M + t, fmaf(al, d, __uint_as_float(rb[t])));
+            v[t] = fmaf(al, d, __uint_as_float(rb[t]));
         }
+        out.put(j * M, v, M);
     }
 }
 
@@ -283,7 +285,11 @@ __device__ __forceinline__ void epilogue_fp4_any_m(const GemmArgs& a, const Unit
 // Cluster form: where a block's partial sums go (its own shared memory, [token][128 weight rows] floats).
 struct FClusterPartOut {
     float* part_row;   // &part[0][this thread's weight row]
-    __device__ __forceinline__ void put(int tok, float v) const { part_row[tok * kTileN] = v; }
+    template <int kTok>
+    __device__ __forceinline__ void put(int tok, const float (&v)[kTok], int) const {
+#pragma unroll
+        for (int t = 0; t < kTok; ++t) part_row[(tok + t) * kTileN] = v[t];
+    }
 };
 
 // The walk over a block's (unit, step) items.  Cluster form (kForm 1): one segment of one unit per block, known without a
@@ -464,7 +470,7 @@ bitdelta_gemm_fp4_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
         mbar_init(smem_u32(&ctl->tmemready), 1);
         mbar_init(smem_u32(&ctl->cntready), 1);
         ctl->abort_flag = 0;
-        ctl->is_last = 0;
+        ctl->npend = 0;
         fence_barrier_init();
     }
     __syncthreads();
@@ -933,7 +939,6 @@ bitdelta_gemm_fp4_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
             }
             if (warp == kFWarpEpi0) FT_STAMP(13);   // counted
         }
-        int pend_unit[2], pend_c0[2], pend_c1[2], npend = 0;   // cut tiles this block has to finish
         // While a tile is being accumulated these four warps prepare every step's activation operands.  Units of up to
         // 16 token rows (a.convert): they write the step's image themselves, one task per thread (fp4_split_task);
         // otherwise the producer's bulk copy brings it.  Either way they then move the image's scale table into
@@ -1073,33 +1078,12 @@ bitdelta_gemm_fp4_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
                 epi_bar_sync(kFEpiWarps * 32);
                 if (*abort_flag) break;
                 if (etid == 0) {
-                    unsigned old;
-                    asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(old) : "l"(a.counters + unit) : "memory");
-                    ctl->is_last = (old == (unsigned)(c1 - c0)) ? 1u : 0u;
-                }
-                epi_bar_sync(kFEpiWarps * 32);
-                if (*abort_flag) break;
-                if (ctl->is_last) {
-                    pend_unit[npend] = unit;
-                    pend_c0[npend] = c0;
-                    pend_c1[npend] = c1;
-                    ++npend;
+                    const unsigned old = atom_add_acq_rel(a.counters + unit);
+                    if (old == (unsigned)(c1 - c0)) ctl->pend_unit[ctl->npend++] = (uint32_t)unit;
                 }
                 FT_ADD(3);
             }
         }
-        // Tiles this block was the last to arrive at (at most its first and its last segment).
-        for (int k = 0; k < npend && ok && !*abort_flag; ++k) {
-            const int un = pend_unit[k], c0 = pend_c0[k], c1 = pend_c1[k];
-            const Unit u = unit_info(a, un);
-            const int first_item = un * a.P;
-            const int slot0 = (cta_first_item(a, c0) == first_item) ? 2 * c0 : 2 * c0 + 1;
-            const float* first = a.partials + (size_t)slot0 * a.slot_floats;
-            const float* rest = a.partials + (size_t)(2 * (c0 + 1)) * a.slot_floats;
-            reduce_partials<false, false>(a, u, etid, kFEpiWarps, first, rest, 2 * (size_t)a.slot_floats, c1 - c0);
-            if (etid == 0) a.counters[un] = 0u;
-        }
-        FT_ADD(4);
         if (warp == kFWarpEpi0) FT_OUT(16, 8);
         if (!ok) {
             // This warp left on an abandoned wait; a sibling that passed the same wait a moment earlier may be
@@ -1124,6 +1108,20 @@ bitdelta_gemm_fp4_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
     }
     tc_fence_after();
     if (warp == kFWarpMma) tmem_dealloc(ctl->tmem_base, kTmemCols);
+    if (kForm != 1 && !*abort_flag) {
+        // Tiles this block was the last to arrive at (at most its first and its last segment).
+        grid_dependency_wait();   // (returns at once: the epilogue warps have passed it)
+        for (int k = 0; k < (int)ctl->npend; ++k) {
+            const int un = (int)ctl->pend_unit[k];
+            const int first_item = un * a.P;
+            const int c0 = cta_of_item(a, first_item), c1 = cta_of_item(a, first_item + a.P - 1);
+            const int slot0 = (cta_first_item(a, c0) == first_item) ? 2 * c0 : 2 * c0 + 1;
+            const float* first = a.partials + (size_t)slot0 * a.slot_floats;
+            const float* rest = a.partials + (size_t)(2 * (c0 + 1)) * a.slot_floats;
+            reduce_partials<false, false>(a, unit_info(a, un), (int)threadIdx.x, kFThreads / 32, first, rest, 2 * (size_t)a.slot_floats, c1 - c0);
+            if (threadIdx.x == 0) a.counters[un] = 0u;
+        }
+    }
     if (is_cluster) {
         // Cluster form: after a cluster barrier the leader's epilogue threads (one weight row each) add the blocks'
         // partial sums in block order, i.e. in k order, through the distributed shared memory window and write Y; a
@@ -1149,10 +1147,10 @@ bitdelta_gemm_fp4_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
                     if (tok + q < u.ntok) {   // (warp-uniform)
-                        float v = reinterpret_cast<const float*>(smem)[(tok + q) * kTileN + row];
+                        float v[1] = {reinterpret_cast<const float*>(smem)[(tok + q) * kTileN + row]};
 #pragma unroll
-                        for (int r = 1; r < 8; ++r) v += pv[q][r];
-                        out.put(tok + q, v);
+                        for (int r = 1; r < 8; ++r) v[0] += pv[q][r];
+                        out.put(tok + q, v, 1);
                     }
                 }
             }

@@ -56,7 +56,7 @@ struct Ctl {
     uint64_t depready;                 // the grid this launch depends on has completed (activations may be read)
     uint32_t tmem_base;
     uint32_t abort_flag;
-    uint32_t is_last;
+    uint32_t npend, pend_unit[2];   // cut tiles this block was the last to arrive at (at most its first and its last)
 };
 static_assert(sizeof(Ctl) <= kSmemCtrlBytes, "control block too large");
 
@@ -122,6 +122,28 @@ bitdelta_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
     const int hi = a.whole_units ? (int)a.T : cta_first_item(a, cta_id + 1);
     SegIter it{lo, hi, a.P, a.whole_units ? (int)gridDim.x : 0};
     int unit, p0, p1;
+
+    // Sums the partial results of a cut tile this block was the last to arrive at.  All warps do it when their roles have
+    // ended; with one or eight tokens per tenant the epilogue warps do it in place (32 x 8 x 14336 x 4096: 155 us, at the end
+    // 170; 16 x 8 x 4096 x 4096: 34.6 and 37.6; but 8 x 12 x 4096 x 4096 29.3 and 26.2, 16 x 4 x 4096 x 11008 with options 66.0
+    // and 64.2: the fix-up's code next to the roles' costs those instantiations more than the shorter tail gains).
+    constexpr bool kEndFixup = kMode != 1 && kMode != 8;
+    auto fix_up = [&](int un, int tid, int n_warps) {
+        // CTA c0 holds the tile's first item; the tile is its first segment only if its range starts exactly there.  Every
+        // later CTA starts inside the tile.
+        // (pair schedule: c0, c1 count clusters; this CTA adds up the slots of the CTAs of its own rank)
+        const int first_item = un * a.P;
+        const int c0 = cta_of_item(a, first_item), c1 = cta_of_item(a, first_item + a.P - 1);
+        const int b0 = kPair ? 2 * c0 + (int)rank : c0;            // first contributing CTA
+        const int bstep = kPair ? 2 : 1;                           // CTAs from one contributor to the next
+        const int slot0 = (cta_first_item(a, c0) == first_item) ? 2 * b0 : 2 * b0 + 1;
+        const float* first = a.partials + (size_t)slot0 * a.slot_floats;
+        const float* rest = a.partials + (size_t)(2 * (b0 + bstep)) * a.slot_floats;
+        const Unit u = unit_info(a, un);
+        if (kGen && a.act == 2) reduce_partials<kGen, kGen>(a, u, tid, n_warps, first, rest, 2 * (size_t)bstep * a.slot_floats, c1 - c0);
+        else reduce_partials<kGen, false>(a, u, tid, n_warps, first, rest, 2 * (size_t)bstep * a.slot_floats, c1 - c0);
+        if (tid == 0) a.counters[kPair ? 2 * un + (int)rank : un] = 0u;
+    };
 
     // Queues the weight loads of one item: its W_base tile into `stage` of the W ring and, if `with_bits`,
     // the sign words of its k-pair into sign-word slot `bslot`.  One thread.
@@ -191,7 +213,7 @@ bitdelta_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
         mbar_init(smem_u32(&ctl->accempty), kDec ? 4 : (kPair ? 16 : 8));
         mbar_init(smem_u32(&ctl->depready), 1);
         ctl->abort_flag = 0;
-        ctl->is_last = 0;
+        ctl->npend = 0;
         fence_barrier_init();
         // The first item's weights are requested right here, before the rest of the CTA is set up:
         // every cycle until the first load is queued is added to the launch's latency.
@@ -915,38 +937,34 @@ bitdelta_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
             }
 
             if (!whole) {
-                // This tile is cut across CTAs: publish the partial, count arrivals, and let
-                // the last CTA to arrive add the partials in CTA order and write Y.
+                // This tile is cut across CTAs: publish the partial and count arrivals.  If this block is the last to arrive it
+                // adds the partials up in CTA order and writes Y.
+                // All epilogue threads' partial stores, then one thread's arrival count: a release over what the barrier ordered
+                // before it, an acquire for what the next barrier orders behind it.
                 const int first_item = unit * a.P;
-                const int c0 = cta_of_item(a, first_item);
-                const int c1 = cta_of_item(a, first_item + a.P - 1);
-                // All epilogue threads' partial stores, then one thread's fence (cumulative over what the
-                // barrier ordered before it) and the arrival count.
+                const int parts = cta_of_item(a, first_item + a.P - 1) - cta_of_item(a, first_item);
                 epi_bar_sync(n_epi_warps * 32);
                 if (*abort_flag) break;   // (a sibling left on an abandoned wait and released this barrier once)
                 if (etid == 0) {
-                    __threadfence();
-                    const unsigned old = atomicAdd(&a.counters[kPair ? 2 * unit + (int)rank : unit], 1u);
-                    ctl->is_last = (old == (unsigned)(c1 - c0)) ? 1u : 0u;
+                    const unsigned old = atom_add_acq_rel(&a.counters[kPair ? 2 * unit + (int)rank : unit]);
+                    if constexpr (!kEndFixup) ctl->npend = (old == (unsigned)parts) ? 1u : 0u;
+                    else if (old == (unsigned)parts) ctl->pend_unit[ctl->npend++] = (uint32_t)unit;
                 }
-                epi_bar_sync(n_epi_warps * 32);
-                if (*abort_flag) break;   // (a sibling left on an abandoned wait and released this barrier once)
-                if (ctl->is_last) {
-                    __threadfence();
-                    // CTA c0 holds the tile's first item; the tile is its first segment only if its
-                    // range starts exactly there.  Every later CTA starts inside the tile.
-                    // (pair schedule: c0, c1 count clusters; this CTA adds up the slots of the CTAs of its own rank)
-                    const int b0 = kPair ? 2 * c0 + (int)rank : c0;            // first contributing CTA
-                    const int bstep = kPair ? 2 : 1;                           // CTAs from one contributor to the next
-                    const int slot0 = (cta_first_item(a, c0) == first_item) ? 2 * b0 : 2 * b0 + 1;
-                    const float* first = a.partials + (size_t)slot0 * a.slot_floats;
-                    const float* rest = a.partials + (size_t)(2 * (b0 + bstep)) * a.slot_floats;
-                    if (kGen && a.act == 2) reduce_partials<kGen, kGen>(a, u, etid, n_epi_warps, first, rest, 2 * (size_t)bstep * a.slot_floats, c1 - c0);
-                    else reduce_partials<kGen, false>(a, u, etid, n_epi_warps, first, rest, 2 * (size_t)bstep * a.slot_floats, c1 - c0);
-                    if (etid == 0) a.counters[kPair ? 2 * unit + (int)rank : unit] = 0u;
+                if constexpr (!kEndFixup) {
+                    epi_bar_sync(n_epi_warps * 32);
+                    if (*abort_flag) break;
+                    if (ctl->npend) {
+                        const int c0 = cta_of_item(a, first_item);
+                        const int slot0 = (cta_first_item(a, c0) == first_item) ? 2 * c0 : 2 * c0 + 1;
+                        const float* first = a.partials + (size_t)slot0 * a.slot_floats;
+                        const float* rest = a.partials + (size_t)(2 * (c0 + 1)) * a.slot_floats;
+                        if (kGen && a.act == 2) reduce_partials<kGen, kGen>(a, u, etid, n_epi_warps, first, rest, 2 * (size_t)a.slot_floats, parts);
+                        else reduce_partials<kGen, false>(a, u, etid, n_epi_warps, first, rest, 2 * (size_t)a.slot_floats, parts);
+                        if (etid == 0) a.counters[unit] = 0u;
+                    }
+                    epi_bar_sync(n_epi_warps * 32);   // npend is rewritten by the next cut tile
+                    if (*abort_flag) break;
                 }
-                epi_bar_sync(n_epi_warps * 32);   // is_last is rewritten by the next cut tile
-                if (*abort_flag) break;   // (a sibling left on an abandoned wait and released this barrier once)
             }
         }
         if (!ok) {
@@ -971,6 +989,10 @@ bitdelta_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
         __syncthreads();
     }
     tc_fence_after();
+    if constexpr (kEndFixup) if (!*abort_flag) {
+        grid_dependency_wait();   // (returns at once: the epilogue warps have passed it)
+        for (int k = 0; k < (int)ctl->npend; ++k) fix_up((int)ctl->pend_unit[k], (int)threadIdx.x, kThreads / 32);
+    }
     if constexpr (kPair) cluster_sync_all();   // neither CTA's shared or tensor memory goes while the other may still signal it
     if (warp == kWarpTmem) {
         if constexpr (kPair) tmem_dealloc_pair(tmem_base, kTmemCols);
