@@ -306,14 +306,14 @@ __device__ __forceinline__ void epilogue_tiled(const GemmArgs& a, const Unit& u,
 }
 
 // Tiled schedule with several tenants per unit (16 < m <= 64): tenant j's base columns start at j*m, its delta
-// columns at j*Nd; 16-token chunks, dealt alternately to the two warps of a lane quadrant.
+// columns at j*Nd; 16-token chunks, one warp per lane quadrant.
 // `al_lane`: lane l holds the scale of the unit's tenant l.
 template <class Out>
 __device__ __forceinline__ void epilogue_tiled_grouped(const GemmArgs& a, const Unit& u, uint32_t lane_taddr, int m,
-                                                       const Out& out, int half, float al_lane) {
+                                                       const Out& out, float al_lane) {
     const int chunks = (m + 15) >> 4;
 #pragma unroll 1
-    for (int c = half; c < u.nten * chunks; c += 2) {
+    for (int c = 0; c < u.nten * chunks; ++c) {
         const int j = c / chunks, t0 = (c - j * chunks) * 16;
         uint32_t rb[16], rd[16];
         tmem_ld16(lane_taddr + (uint32_t)(j * m + t0), rb);

@@ -37,7 +37,7 @@ constexpr int kWarpTmem = 2;
 constexpr int kWarpDelta0 = 2;     // decode schedule: warps 2..3 issue the delta MMAs of decode group 0 / 1
 constexpr int kBarAFull0 = 2;      // named barriers 2..9 : decode group g, buffer b -> id 2 + g*4 + b
 constexpr int kWarpDecode0 = 4;    // warps 4..11
-constexpr int kRaggedBitThreads = 64;   // tiled schedule, K % 128 != 0: warps 2..3 copy the sign words
+constexpr int kRaggedBitThreads = 64;   // tiled schedule, K % 128 != 0: two warps copy the sign words (2..3, or two more with several tenants per unit)
 constexpr int kWarpEpi0 = 12;      // warps 12..15
 
 struct Ctl {
@@ -68,8 +68,9 @@ static_assert(sizeof(Ctl) <= kSmemCtrlBytes, "control block too large");
 // kGen: the general form (binary16 I/O, bias, activation); false compiles the plain bf16 product alone, whose
 // code is then exactly as short as it can be (the kernel's speed is sensitive to its length).
 // kRagged: K % 128 != 0 (tiled modes, general form); a form of its own because the run-time test cost the others 2 %.
+__host__ __device__ constexpr int threads_of(int mode, bool ragged) { return kThreads + (mode == 6 && ragged ? kRaggedBitThreads : 0); }
 template <int kMode, bool kGen, bool kRagged = false>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(threads_of(kMode, kRagged), 1)
 bitdelta_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX,
                         const __grid_constant__ CUtensorMap tmX8, const __grid_constant__ CUtensorMap tmBits,
                         const GemmArgs a) {
@@ -91,6 +92,11 @@ bitdelta_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
     constexpr bool kGrouped = kMode == 6;   // tiled schedule with several tenants per unit (16 < m <= 64)
     constexpr bool kPair = kMode == 7;      // tiled schedule on CTA pairs (cluster of two, 256-row MMAs)
     constexpr bool kDec = (kMode >= 1 && kMode <= 5) || kMode == 8;
+    // Three MMA issuers (base; delta of the even / of the odd tenants) and two decode groups of four warps: the decode
+    // schedules, and the tiled one with several tenants per unit, where a step is 8 base and 8 narrow delta MMAs per tenant
+    // and one thread issues one of them per ~48 cycles whatever their width (8 x 32 x 4096 x 4096: 39.7 us with one issuer
+    // and four decode warps, 29.9 now; 8 x 64: 46.3 and 36.6).
+    constexpr bool kSplit = kDec || kGrouped;
     // Pair schedule: this CTA's rank in its cluster (0 = leader, issues the MMAs), the leader's view of
     // the barriers both CTAs signal, and the work share of the CLUSTER.
     const uint32_t rank = kPair ? cluster_ctarank() : 0u;
@@ -106,10 +112,11 @@ bitdelta_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
     auto unit_info = [&](const GemmArgs& aa, int un) { return unit_info_t<kDec, kGrouped, kPair>(aa, un, am, (int)rank); };
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
-    // Tiled schedule: signs need few decode threads, the epilogue many -> warps 8..11 drain accumulators
-    // instead of decoding.
-    constexpr int epi_first_warp = kDec ? kWarpEpi0 : kWarpEpi0 - 4;
+    // Tiled schedule, one tenant per unit: signs need few decode threads, the epilogue many -> warps 8..11 drain
+    // accumulators instead of decoding.
+    constexpr int epi_first_warp = kSplit ? kWarpEpi0 : kWarpEpi0 - 4;
     constexpr int n_epi_warps = 16 - epi_first_warp;
+    constexpr int kWarpBits0 = kGrouped ? 16 : kWarpDelta0;   // K % 128 != 0: the two warps that copy the sign words
     if (threadIdx.x == 32) {
         prefetch_tensormap(&tmW);
         prefetch_tensormap(&tmX);
@@ -197,7 +204,7 @@ bitdelta_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
     if (threadIdx.x == 0) {
         for (int s = 0; s < kMaxStages; ++s) {
             mbar_init(smem_u32(&ctl->wfull[s]), 1);
-            mbar_init(smem_u32(&ctl->wempty[s]), 1);
+            mbar_init(smem_u32(&ctl->wempty[s]), kGrouped ? 3 : 1);              // (several tenants: the three issuers)
             mbar_init(smem_u32(&ctl->xfull[s]), 1);
             mbar_init(smem_u32(&ctl->xempty[s]), (kDec && convert) ? 129 : 1);   // base issuer (+ the splitter threads)
             mbar_init(smem_u32(&ctl->x8full[s]), (kDec && convert) ? 128 : 1);   // splitter threads, or one TMA load
@@ -205,12 +212,12 @@ bitdelta_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
         }
         for (int s = 0; s < kMaxBitSlots; ++s) {
             mbar_init(smem_u32(&ctl->bfull[s]), ragged ? kRaggedBitThreads : 1);   // (ragged: every copying thread)
-            mbar_init(smem_u32(&ctl->bempty[s]), kDec ? 8 : 4);
+            mbar_init(smem_u32(&ctl->bempty[s]), kSplit ? 8 : 4);
         }
         for (int s = 0; s < kMaxASlots; ++s) mbar_init(smem_u32(&ctl->afull[s]), kPair ? 8 : 4);   // (pair: both CTAs' decode warps)
         for (int s = 0; s < 2 * kMaxASlots; ++s) mbar_init(smem_u32(&ctl->aempty[s]), 1);
-        mbar_init(smem_u32(&ctl->accfull), kDec ? 3 : 1);
-        mbar_init(smem_u32(&ctl->accempty), kDec ? 4 : (kPair ? 16 : 8));
+        mbar_init(smem_u32(&ctl->accfull), kSplit ? 3 : 1);
+        mbar_init(smem_u32(&ctl->accempty), kSplit ? 4 : (kPair ? 16 : 8));
         mbar_init(smem_u32(&ctl->depready), 1);
         ctl->abort_flag = 0;
         ctl->npend = 0;
@@ -457,14 +464,16 @@ bitdelta_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
                                     idesc_base, (kk > 0) ? 1u : first);
                     }
                     // decode schedule: nothing else reads the W_base tile, hand it back as soon as these MMAs
-                    // have completed
+                    // have completed (several tenants: one of the stage's three releases)
                     if (kDec) {
                         tc_commit(smem_u32(&ctl->wempty[stage]));
                         tc_commit(smem_u32(&ctl->xempty[xslot]));
+                    } else if (kGrouped) {
+                        tc_commit(smem_u32(&ctl->wempty[stage]));
                     }
                 }
                 __syncwarp();
-                if constexpr (kDec) {
+                if constexpr (kSplit) {
                     // Delta MMAs are issued by the two delta-issuer warps.
                 } else {
                     for (int j = 0; j < u.nten && ok; ++j, ++item, ar.step()) {
@@ -493,7 +502,7 @@ bitdelta_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
                     }
                 }
                 if (!ok) break;
-                if (!kDec) {
+                if (!kSplit) {
                     if (elect_one()) {
                         if constexpr (kPair) tc_commit_pair(smem_u32(&ctl->wempty[stage]), 3);
                         else tc_commit(smem_u32(&ctl->wempty[stage]));
@@ -511,7 +520,7 @@ bitdelta_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
             __syncwarp();
             accphase ^= 1;
         }
-    } else if (warp >= kWarpDelta0 && warp < kWarpDelta0 + 2) {
+    } else if (warp >= kWarpDelta0 && warp < kWarpDelta0 + 2 && (kSplit || !ragged)) {
         // ------------------------------------------------- delta issuers (decode schedule)
         // Warp 2+g serves decode group g (tenants j = g, g+2, ... of the unit).  Per 128-k stage it
         //  * waits for the stage's e5m2 piece tile, and
@@ -585,13 +594,62 @@ bitdelta_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
                 __syncwarp();
                 accphase ^= 1;
             }
-        } else if (ragged) {
+        } else if constexpr (kGrouped) {
+            // ... tiled schedule, several tenants per unit: warp 2+g serves the tenants j = g, g+2, ..., one operand buffer
+            // (a tenant's signs of 128 k) per hand-over; the activation tile lives in the W_base stage.
+            const int g = warp - kWarpDelta0;
+            const uint32_t idesc_delta = io_f16 ? make_idesc_f16(kTileN, (uint32_t)a.Nd) : make_idesc_bf16(kTileN, (uint32_t)a.Nd);
+            const uint64_t desc0 = make_smem_desc_sw128(0);
+            const uint32_t x_atom16 = a.x_atom_bytes >> 4;
+            Ring ar{0, 0u, a.a_slots};   // this group's operand buffers in tensor memory
+            int stage = 0;
+            uint32_t phase = 0, accphase = 0;
+            bool ok = true;
+            while (ok && it.next(unit, p0, p1)) {
+                const Unit u = unit_info(a, unit);
+                ok = warp_all(wait_bar(smem_u32(&ctl->accempty), accphase ^ 1, abort_flag, 3));
+                if (!ok) break;
+                tc_fence_after();
+                for (int p = p0; p < p1 && ok; ++p) {
+                    ok = warp_all(wait_bar(smem_u32(&ctl->wfull[stage]), phase, abort_flag, 4));
+                    if (!ok) break;
+                    const uint64_t xdesc = desc0 + ((x_addr + stage * a.x_tile_bytes) >> 4);
+                    const uint32_t first = (p > p0) ? 1u : 0u;   // 0: this step starts the accumulation
+                    for (int j = g; j < u.nten; j += 2, ar.step()) {
+                        if (*abort_flag) { ok = false; break; }
+                        named_bar_sync(kBarAFull0 + g * 4 + ar.idx, 160);   // filled by the group's 128 decode threads
+                        if (*abort_flag) { ok = false; break; }
+                        tc_fence_after();
+                        const uint32_t d_tmem = tmem_base + a.col_delta + (uint32_t)(j * a.Nd);
+                        const uint32_t a_tmem = tmem_base + a.col_a + (uint32_t)(g * a.a_slots + ar.idx) * (uint32_t)a.aslot_cols;
+                        const uint64_t xj = xdesc + (uint32_t)(j * a.win_rows) * 8u;   // 128 B per row
+                        if (elect_one()) {
+#pragma unroll
+                            for (int kk = 0; kk < 8; ++kk)
+                                umma_ts(d_tmem, a_tmem + kk * 8, xj + ((kk >> 2) * x_atom16 + (kk & 3) * 2), idesc_delta, (kk > 0) ? 1u : first);
+                            tc_commit(smem_u32(&ctl->aempty[g * kMaxASlots + ar.idx]));
+                        }
+                        __syncwarp();
+                    }
+                    if (!ok) break;
+                    if (elect_one()) tc_commit(smem_u32(&ctl->wempty[stage]));
+                    __syncwarp();
+                    if (++stage == a.n_w) { stage = 0; phase ^= 1; }
+                }
+                if (!ok) break;
+                if (elect_one()) tc_commit(smem_u32(&ctl->accfull));
+                __syncwarp();
+                accphase ^= 1;
+            }
+        }
+    } else if (ragged && warp >= kWarpBits0 && warp < kWarpBits0 + 2) {
+        if constexpr (ragged) {
             // ------------------------------------------- sign words (tiled schedule, K % 128 != 0)
             // The row pitch of the sign words is a multiple of 4 bytes only, so no tensor map takes them: these two
-            // otherwise idle warps copy them word by word into the slots (eight consecutive lanes take the eight words
+            // warps, which have nothing else to do, copy them word by word into the slots (eight consecutive lanes take the eight words
             // of a row: 32 contiguous bytes), as far ahead as the ring allows.  Words past the row's end and
             // rows past N are zero-filled; the zero-filled activations of the short step make them count for nothing.
-            const int btid = (int)threadIdx.x - kWarpDelta0 * 32;
+            const int btid = (int)threadIdx.x - kWarpBits0 * 32;
             const int words = a.K >> 5;
             ItemIter bi(it);
             int bslot = 0;
@@ -743,6 +801,25 @@ bitdelta_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
                         tc_fence_before();
                         named_bar_arrive(kBarAFull0 + grp * 4 + (int)slot, 160);
                     }
+                } else if constexpr (kGrouped) {
+                    // warp (grp, quad): the tenants j = grp, grp+2, ..., one buffer of the group's ring each
+                    for (int j = grp; j < u.nten && ok; j += 2, ar.step()) {
+                        const uint4 w = *reinterpret_cast<const uint4*>(bsl + (j * kTileN + row) * 32);
+                        uint32_t r[32], r2[32];
+                        decode_word(w.x, r, minus_one2);
+                        decode_word(w.y, r + 16, minus_one2);
+                        ok = wait_bar(aempty_g + (uint32_t)ar.idx * 8, ar.par ^ 1, abort_flag, 7);
+                        if (!ok) break;
+                        tc_fence_after();
+                        const uint32_t tbuf = tbuf_g + (uint32_t)ar.idx * (uint32_t)a.aslot_cols;
+                        tmem_st32(tbuf, r);
+                        decode_word(w.z, r2, minus_one2);
+                        decode_word(w.w, r2 + 16, minus_one2);
+                        tmem_st32(tbuf + 32, r2);
+                        tc_wait_st();
+                        tc_fence_before();
+                        named_bar_arrive(kBarAFull0 + grp * 4 + ar.idx, 160);
+                    }
                 } else {
                     for (int j = 0; j < u.nten && ok; ++j, ++item, ar.step()) {
                         const uint4 w = *reinterpret_cast<const uint4*>(bsl + (j * kTileN + row) * 32);
@@ -775,14 +852,14 @@ bitdelta_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
                 }
             }
         }
-        if (kDec && *abort_flag) {
+        if (kSplit && *abort_flag) {
             // A wait was abandoned somewhere in the CTA.  The group's delta issuer may be blocked on one
             // of the named barriers (they have no time-out): arrive on all of them so that it wakes up,
             // sees the abort flag and leaves.
             __syncwarp();
             for (int sl = 0; sl < a.a_slots; ++sl) named_bar_arrive(kBarAFull0 + grp * 4 + sl, 160);
         }
-    } else if (warp >= epi_first_warp) {
+    } else if (warp >= epi_first_warp && warp < 16) {
         // ---------------------------------------------------------------- epilogue
         const int quad = warp & 3;
         const int row = quad * 32 + lane;
@@ -919,7 +996,7 @@ bitdelta_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
                         default: epilogue_decode<16, kGen>(a, u, lane_taddr, out, alv, al_lane); break;
                     }
                 } else {
-                    if constexpr (kGrouped) epilogue_tiled_grouped(a, u, lane_taddr, am, out, ehalf, al_lane);
+                    if constexpr (kGrouped) epilogue_tiled_grouped(a, u, lane_taddr, am, out, al_lane);
                     else epilogue_tiled(a, u, lane_taddr, out, ehalf, alv[0], release_acc);
                 }
             };
@@ -991,7 +1068,7 @@ bitdelta_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
     tc_fence_after();
     if constexpr (kEndFixup) if (!*abort_flag) {
         grid_dependency_wait();   // (returns at once: the epilogue warps have passed it)
-        for (int k = 0; k < (int)ctl->npend; ++k) fix_up((int)ctl->pend_unit[k], (int)threadIdx.x, kThreads / 32);
+        for (int k = 0; k < (int)ctl->npend; ++k) fix_up((int)ctl->pend_unit[k], (int)threadIdx.x, threads_of(kMode, kRagged) / 32);
     }
     if constexpr (kPair) cluster_sync_all();   // neither CTA's shared or tensor memory goes while the other may still signal it
     if (warp == kWarpTmem) {
@@ -1032,7 +1109,7 @@ cudaError_t launch_gemm_tc(const CUtensorMap& tmW, const CUtensorMap& tmX, const
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3((unsigned)threads_of(mode == 19 ? 6 : 0, mode == 19));
     cfg.dynamicSmemBytes = smem_bytes;
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];

@@ -397,7 +397,7 @@ inline Plan make_plan(int B, int m, int N, int K, int num_sms, int tb_override =
         p.aslot_cols *= 2;
     }
     int slots = free_cols / p.aslot_cols;
-    if (p.decode) slots /= 2;                          // each of the two decode groups has its own ring
+    if (p.decode || p.win_rows > 0) slots /= 2;        // two decode groups, each with its own ring (also several tenants per tiled unit)
     p.a_slots = slots >= 4 ? 4 : slots >= 2 ? 2 : 0;   // power of two
     if (p.a_slots > kMaxASlots) p.a_slots = kMaxASlots;
     if (p.fp4) {
