@@ -13,6 +13,7 @@ _HERE = os.path.dirname(os.path.abspath(__file__))
 # BITDELTA_LIB points at another build of the same library (the trace build made by `build.py --trace`).
 _LIB_PATH = os.environ.get("BITDELTA_LIB") or os.path.join(_HERE, "libbitdelta.so")
 _lib = None
+_fast = None      # the extension module's `gemm`, once the library is loaded (see csrc/fastcall.cpp)
 
 STATUS_OK = 0
 STATUS_TIMEOUT = 7
@@ -40,7 +41,7 @@ def library_path() -> str:
 
 def load_library():
     """Load libbitdelta.so (built in-tree by paper_2609_36800_b200.build); raises if absent."""
-    global _lib
+    global _lib, _fast
     if _lib is not None:
         return _lib
     if not os.path.exists(_LIB_PATH):
@@ -75,6 +76,13 @@ def load_library():
     for fn in ("bitdelta_pack", "bitdelta_unpack", "bitdelta_compress", "bitdelta_workspace_init", "bitdelta_gemm",
                "bitdelta_gemm_simt", "bitdelta_gemm_noalloc", "bitdelta_gemm_host", "bitdelta_last_device_status"):
         getattr(lib, fn).restype = ci
+    try:
+        import torch   # noqa: F401  (the extension module links against its libraries)
+        from . import _fastcall
+        _fastcall.set_library(ctypes.cast(lib.bitdelta_gemm_ex, vp).value)
+        _fast = _fastcall.gemm
+    except ImportError:   # (not built against this torch: every call goes through the checks below)
+        _fast = None
     _lib = lib
     return lib
 
@@ -176,6 +184,11 @@ def gemm(X, W_base, bits, alpha, out=None, workspace=None, stream=None, simt: bo
     returns Y [B,m,N] of X's type.  wide_range=True plans every m on the tiled schedule (for activations of
     magnitude 2^16 or more, which the decode schedules clamp and flag).  (simt=True runs the diagnostic
     CUDA-core kernel: bf16, no epilogue.)"""
+    if _fast is not None and out is not None and workspace is not None and stream is None and not simt and act in ACTS:
+        st = _fast(X, W_base, bits, alpha, bias, out, workspace, DTYPE_WIDE_RANGE if wide_range else 0, ACTS[act])
+        if st == STATUS_OK:
+            return out
+        # (another status: the same call below raises it under the entry point's name)
     import torch
     lib = load_library()
     B, m, K = X.shape

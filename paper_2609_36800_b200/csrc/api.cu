@@ -192,14 +192,19 @@ struct MapKey {
         return kind == o.kind && ptr == o.ptr && d0 == o.d0 && d1 == o.d1 && d2 == o.d2 && b0 == o.b0 && b1 == o.b1;
     }
 };
-constexpr int kMapCacheSize = 64;
+// (a table of sets of four by a hash of the key, so that a look-up compares four keys however many are held)
+constexpr int kMapSets = 64, kMapWays = 4;
 struct MapCache {
     std::mutex mu;
-    MapKey keys[kMapCacheSize];
-    CUtensorMap maps[kMapCacheSize];
-    bool used[kMapCacheSize] = {};
-    int next = 0;
+    MapKey keys[kMapSets][kMapWays];
+    CUtensorMap maps[kMapSets][kMapWays];
+    uint8_t used[kMapSets] = {}, next[kMapSets] = {};
 };
+inline unsigned map_set(const MapKey& k) {
+    uint64_t h = reinterpret_cast<uint64_t>(k.ptr) ^ (k.d0 * 0x9E3779B97F4A7C15ull) ^ (k.d1 << 20) ^ ((uint64_t)k.b0 << 44) ^ ((uint64_t)k.kind << 60);
+    h *= 0x9E3779B97F4A7C15ull;
+    return (unsigned)(h >> 58);   // 64 sets
+}
 MapCache& map_cache() {
     static MapCache c;
     return c;
@@ -207,21 +212,22 @@ MapCache& map_cache() {
 template <class Encode>
 bool cached_map(CUtensorMap* out, const MapKey& key, Encode encode) {
     MapCache& c = map_cache();
+    const unsigned s = map_set(key);
     {
         std::lock_guard<std::mutex> lock(c.mu);
-        for (int i = 0; i < kMapCacheSize; ++i)
-            if (c.used[i] && c.keys[i] == key) {
-                *out = c.maps[i];
+        for (int i = 0; i < c.used[s]; ++i)
+            if (c.keys[s][i] == key) {
+                *out = c.maps[s][i];
                 return true;
             }
     }
     if (!encode(out)) return false;
     std::lock_guard<std::mutex> lock(c.mu);
-    const int i = c.next;
-    c.next = (c.next + 1) % kMapCacheSize;
-    c.keys[i] = key;
-    c.maps[i] = *out;
-    c.used[i] = true;
+    const int i = c.next[s];
+    c.next[s] = (uint8_t)((i + 1) % kMapWays);
+    if (c.used[s] <= i) c.used[s] = (uint8_t)(i + 1);
+    c.keys[s][i] = key;
+    c.maps[s][i] = *out;
     return true;
 }
 
