@@ -293,6 +293,10 @@ size_t bitdelta_gemm_workspace_bytes(int B, int m, int N, int K) {
     if ((K % 128) != 0 && !p.ok) return 256;   // CUDA-core path: no scratch needed, keep the pointer non-NULL
     if (!p.ok) return 0;
     size_t need = p.ws_bytes;
+    if (p.pair) {   // ... and without pairs, for a device (or a part of one) that cannot hold them all at once
+        bd::Plan o = bd::make_plan(B, m, N, K, 148, tb_override(), whole_override(), false);
+        if (o.ok && o.ws_bytes > need) need = o.ws_bytes;
+    }
     if (p.decode) {   // the same shape on the tiled schedule (BITDELTA_DTYPE_WIDE_RANGE) may need more
         bd::Plan w = bd::make_plan(B, m, N, K, 148, tb_override(), whole_override(), true, true);
         if (w.ok && w.ws_bytes > need) need = w.ws_bytes;

@@ -158,7 +158,8 @@ __device__ __forceinline__ void tmem_ld_w(uint32_t taddr, uint32_t* r) {
     else if constexpr (W == 2) tmem_ld2(taddr, r);
     else if constexpr (W == 4) tmem_ld4(taddr, r);
     else if constexpr (W == 8) tmem_ld8(taddr, r);
-    else tmem_ld16(taddr, r);
+    else if constexpr (W == 16) tmem_ld16(taddr, r);
+    else tmem_ld32(taddr, r);
 }
 
 // Fused epilogue on a finished sum: bias, then the activation, then rounding to the I/O type.
@@ -182,6 +183,7 @@ __device__ __forceinline__ float from_io16(uint16_t h, int f16) {
 // product should not pay for the general form's length.
 template <bool kGen, bool kGate = false>
 struct EpiOut {
+    static constexpr bool kGeneral = kGen;
     uint16_t* Y;        // output matrix [B*m, N], 16-bit values of the I/O type
     float* slot;        // partial-result slot, or nullptr when this CTA owns the whole tile
     int N, n, row, xrow0;
@@ -200,34 +202,40 @@ struct EpiOut {
                 if (t < nvalid) p[t * kTileN] = v[t];
             return;
         }
+        uint32_t o[(kTok + 1) / 2];
+        finish(v, o);
+        store<kTok>(tok, o, nvalid);
+    }
+    // ... in two parts: the results in the I/O type, two token rows per register, and their stores to Y.
+    template <int kTok>
+    __device__ __forceinline__ void finish(const float (&v)[kTok], uint32_t (&o)[(kTok + 1) / 2]) const {
+        uint16_t h[kTok];
         if constexpr (kGate) {
             // SiLU gate: weight rows come in pairs (2i: gate, 2i+1: up), i.e. in neighbouring lanes
-            const int lim = (!(n & 1) && n < N) ? nvalid : 0;
-            uint16_t* p = Y + (size_t)(xrow0 + tok) * (N >> 1) + (n >> 1);
 #pragma unroll
             for (int t = 0; t < kTok; ++t) {
                 const float z = v[t] + bias;
                 const float other = __shfl_xor_sync(0xFFFFFFFFu, z, 1);
-                const uint16_t o = to_io16(__fdividef(z, 1.f + __expf(-z)) * other, a.f16);
-                if (t < lim) p[(size_t)t * (N >> 1)] = o;
+                h[t] = to_io16(__fdividef(z, 1.f + __expf(-z)) * other, a.f16);
             }
+        } else if (kGen && a.act == 1) {
+#pragma unroll
+            for (int t = 0; t < kTok; ++t) h[t] = finish_io16(v[t], bias, 1, a.f16);
         } else {
-            const int lim = n < N ? nvalid : 0;
-            uint16_t* p = Y + (size_t)(xrow0 + tok) * N + n;
-            if (kGen && a.act == 1) {
 #pragma unroll
-                for (int t = 0; t < kTok; ++t) {
-                    const uint16_t o = finish_io16(v[t], bias, 1, a.f16);
-                    if (t < lim) p[(size_t)t * N] = o;
-                }
-            } else {
-#pragma unroll
-                for (int t = 0; t < kTok; ++t) {
-                    const uint16_t o = kGen ? to_io16(v[t] + bias, a.f16) : __bfloat16_as_ushort(__float2bfloat16_rn(v[t]));
-                    if (t < lim) p[(size_t)t * N] = o;
-                }
-            }
+            for (int t = 0; t < kTok; ++t) h[t] = kGen ? to_io16(v[t] + bias, a.f16) : __bfloat16_as_ushort(__float2bfloat16_rn(v[t]));
         }
+#pragma unroll
+        for (int t = 0; t < kTok; t += 2) o[t / 2] = (uint32_t)h[t] | ((t + 1 < kTok) ? (uint32_t)h[t + 1 < kTok ? t + 1 : t] << 16 : 0u);
+    }
+    template <int kTok>
+    __device__ __forceinline__ void store(int tok, const uint32_t (&o)[(kTok + 1) / 2], int nvalid) const {
+        const int lim = (n < N && !(kGate && (n & 1))) ? nvalid : 0;
+        const int pitch = kGate ? N >> 1 : N;
+        uint16_t* p = Y + (size_t)(xrow0 + tok) * pitch + (kGate ? n >> 1 : n);
+#pragma unroll
+        for (int t = 0; t < kTok; ++t)
+            if (t < lim) p[(size_t)t * pitch] = (uint16_t)(o[t / 2] >> (16 * (t & 1)));
     }
 };
 
@@ -291,17 +299,51 @@ __device__ __forceinline__ void epilogue_decode(const GemmArgs& a, const Unit& u
 template <class Out, class Release>
 __device__ __forceinline__ void epilogue_tiled(const GemmArgs& a, const Unit& u, uint32_t lane_taddr,
                                                const Out& out, int half, float al, const Release& release) {
-    if (32 * half >= u.ntok) release();
-    for (int t0 = 32 * half; t0 < u.ntok; t0 += 64) {
-        uint32_t rb[32], rd[32];
-        tmem_ld32(lane_taddr + (uint32_t)t0, rb);
-        tmem_ld32(lane_taddr + a.col_delta + (uint32_t)t0, rd);
-        tc_wait_ld();
-        if (t0 + 64 >= u.ntok) release();
-        float v[32];
+    if (out.slot) {
+        if (32 * half >= u.ntok) release();
+        for (int t0 = 32 * half; t0 < u.ntok; t0 += 64) {
+            uint32_t rb[32], rd[32];
+            tmem_ld32(lane_taddr + (uint32_t)t0, rb);
+            tmem_ld32(lane_taddr + a.col_delta + (uint32_t)t0, rd);
+            tc_wait_ld();
+            if (t0 + 64 >= u.ntok) release();
+            float v[32];
 #pragma unroll
-        for (int t = 0; t < 32; ++t) v[t] = fmaf(al, __uint_as_float(rd[t]), __uint_as_float(rb[t]));
-        out.put(t0, v, u.ntok - t0);
+            for (int t = 0; t < 32; ++t) v[t] = fmaf(al, __uint_as_float(rd[t]), __uint_as_float(rb[t]));
+            out.put(t0, v, u.ntok - t0);
+        }
+        return;
+    }
+    // A whole tile: the results are held two per register until the accumulators have gone back, then stored (the 2-byte
+    // stores of 128 tokens take 3.8 us, in which the next tile's MMAs run).
+    uint32_t o[kMaxTokTile / 64][16];
+#pragma unroll
+    for (int i = 0; i < kMaxTokTile / 64; ++i) {
+        if (32 * half + 64 * i < u.ntok) {   // (warp-uniform)
+            // (general form: sixteen tokens at a time, which keeps it within the registers)
+            constexpr int kTok = Out::kGeneral ? 16 : 32;
+#pragma unroll
+            for (int c = 0; c < 32; c += kTok) {
+                uint32_t rb[kTok], rd[kTok];
+                const uint32_t col = (uint32_t)(32 * half + 64 * i + c);
+                tmem_ld_w<kTok>(lane_taddr + col, rb);
+                tmem_ld_w<kTok>(lane_taddr + a.col_delta + col, rd);
+                tc_wait_ld();
+                float v[kTok];
+                uint32_t oc[kTok / 2];
+#pragma unroll
+                for (int t = 0; t < kTok; ++t) v[t] = fmaf(al, __uint_as_float(rd[t]), __uint_as_float(rb[t]));
+                out.finish(v, oc);
+#pragma unroll
+                for (int t = 0; t < kTok / 2; ++t) o[i][c / 2 + t] = oc[t];
+            }
+        }
+    }
+    release();
+#pragma unroll
+    for (int i = 0; i < kMaxTokTile / 64; ++i) {
+        const int t0 = 32 * half + 64 * i;
+        if (t0 < u.ntok) out.template store<32>(t0, o[i], u.ntok - t0);
     }
 }
 

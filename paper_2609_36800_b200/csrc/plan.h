@@ -18,6 +18,7 @@ constexpr int kMaxASlots = 4;
 constexpr int kPieces = 4;           // e5m2 pieces an activation is split into for the decode-regime delta MMA
 constexpr int kTmemCols = 512;
 constexpr int kMaxCtas = 256;        // upper bound on the grid, sizes the workspace
+constexpr int kMaxTokTile = 192;      // tokens of a tiled unit, at most (CTA pairs; 128 otherwise)
 constexpr int kDecodeMaxM = 16;      // m <= 16: tenants are grouped into one tile
 constexpr int kSmemBudget = 227 * 1024;
 constexpr int kSmemCtrlBytes = 1024; // barriers, TMEM base, flags
@@ -193,14 +194,21 @@ inline Plan make_plan(int B, int m, int N, int K, int num_sms, int tb_override =
         p.slot_floats = (size_t)kTileN * p.TB * m;
     } else {
         p.TB = 1;
-        p.tok_tile = m >= 128 ? 128 : round_up(m, 16);
+        // CTA pairs take up to 192 tokens a tile (two operand buffers are left beside 384 accumulator columns), single blocks
+        // 128; a tenant's tokens are spread evenly over its tiles.  The tiles' loads from L2 weigh on the schedule (31 bytes per
+        // cycle and multiprocessor at 128 tokens), and a half-empty last tile costs as much as a full one: 4 x 512 x 4096 x
+        // 4096 in tiles of 128: 103.5 us, of 176: 97.7; 4 x 130: 53.4 (two of 128) and 34.5 (one of 144); 2 x 300 x 4096 x
+        // 11008 binary16 with a gate: 115.9 (three of 128) and 97.6 (two of 160).
+        const bool pairs = allow_pair && pair_enabled() && m > 64 && (p.n_tiles % 2) == 0 && num_sms >= 2;
+        p.m_tiles = (m + (pairs ? kMaxTokTile : 128) - 1) / (pairs ? kMaxTokTile : 128);
+        p.tok_tile = round_up((m + p.m_tiles - 1) / p.m_tiles, 16);
         p.m_tiles = (m + p.tok_tile - 1) / p.tok_tile;
         p.groups = B * p.m_tiles;
         p.Nb = p.tok_tile;
         p.Nd = p.tok_tile;
         p.win_rows = 0;
         p.chunk_rows = 16;
-        p.pair = (allow_pair && pair_enabled() && p.tok_tile >= 80 && (p.n_tiles % 2) == 0 && num_sms >= 2) ? 1 : 0;
+        p.pair = (pairs && p.tok_tile >= 80) ? 1 : 0;
         p.x_rows = p.pair ? p.tok_tile / 2 : p.tok_tile;   // a pair's CTAs stage half of the token tile each
         p.N3 = 0;
         p.convert = 0;
@@ -372,6 +380,11 @@ inline Plan make_plan(int B, int m, int N, int K, int num_sms, int tb_override =
     } else {
         p.n_x8 = 0;
         p.n_w = avail / (int)(p.w_stage_bytes + p.x_tile_bytes);
+        // (half of the sign-word ring goes where that makes room for another stage)
+        if (p.n_bits > 4 && (avail + (p.n_bits - 4) * (int)p.bslot_bytes) / (int)(p.w_stage_bytes + p.x_tile_bytes) > p.n_w) {
+            p.n_bits = 4;
+            ++p.n_w;
+        }
         if (p.n_w > kMaxStages) p.n_w = kMaxStages;
         p.n_x = p.n_w;
     }
