@@ -398,6 +398,8 @@ def kernels_per_step(wl):
     pre-pass kernel in the 4-bit decode schedule and in the 8-bit decode schedule with more than 16 token rows per
     unit (otherwise the GEMM kernel splits the activations itself)."""
     import paper_2609_36800_b200 as bd
+    if bd.gemm_row_stream(wl.B, wl.m, wl.N, wl.K):
+        return 1
     schedule = bd.gemm_plan(wl.B, wl.m, wl.N, wl.K)["schedule"]
     if schedule in (7, 8):
         return 1 if os.environ.get("BITDELTA_FP4_INKERNEL") else 2
@@ -406,6 +408,8 @@ def kernels_per_step(wl):
 
 def gemm_kernel_name(wl):
     import paper_2609_36800_b200 as bd
+    if bd.gemm_row_stream(wl.B, wl.m, wl.N, wl.K):
+        return "bitdelta_gemm_row_kernel"
     schedule = bd.gemm_plan(wl.B, wl.m, wl.N, wl.K)["schedule"]
     return {7: "bitdelta_gemm_fp4_kernel", 8: "bitdelta_gemm_fp4_kernel", 3: "gemm_simt_kernel"}.get(schedule, "bitdelta_gemm_tc_kernel")
 

@@ -110,7 +110,9 @@ int bitdelta_workspace_init(void* workspace, size_t workspace_bytes, void* cuda_
  * X, W_base, bits and Y must be 16-byte aligned; K a multiple of 32.
  * Asynchronous on the stream; a kernel-side wait that expires is reported by
  * bitdelta_last_device_status, not here.
- * Precision of X in the decode schedules (m <= 16): there the delta term runs on
+ * Row-stream shapes (bitdelta_gemm_row_stream; m <= 8) keep X as it is in both terms and
+ * take any magnitude.
+ * Precision of X in the decode schedules (other m <= 16): there the delta term runs on
  * a narrow-float tensor path.  bitdelta_gemm_plan tells which of two a shape gets.
  * 4-bit schedules (plan codes 7, 8; m <= 8, calls without options): every group
  * of 32 consecutive k of a token row is held as 16-bit fixed point relative to the
@@ -231,6 +233,10 @@ int bitdelta_gemm_host(const void* X_host, const void* W_base_host, const uint32
  * is one 128-row tile of W_base for one group of TB tenants (decode schedules) or one tenant's token tile
  * (tiled schedule), a k-step is 128 k; item = unit * P + k-step.
  *
+ * bitdelta_gemm_row_stream returns 1 for the shapes (few tenants, or small; m <= 8) that run on the row-stream kernel instead: one
+ * launch, no scratch, a block per few weight rows with all of K.  bitdelta_gemm_plan reports the schedule that it stands
+ * in for, which the same call takes with BITDELTA_ROW=0 in the environment.
+ *
  * bitdelta_gemm_plan fills info[0 .. BITDELTA_PLAN_INFO_INTS-1] (host pointer):
  *   [0] schedule: 0 tiled, 1 decode with a pre-pass activation split, 2 decode with the in-kernel split,
  *       3 CUDA-core kernel (K not a multiple of 128 and a small product; all other entries are 0 then), 4 tiled on pairs of
@@ -255,6 +261,7 @@ int bitdelta_gemm_host(const void* X_host, const void* W_base_host, const uint32
  */
 #define BITDELTA_PLAN_INFO_INTS 16
 int bitdelta_gemm_plan(int B, int m, int N, int K, int num_sms, int* info);
+int bitdelta_gemm_row_stream(int B, int m, int N, int K, int num_sms);
 int bitdelta_gemm_plan_cta_items(int B, int m, int N, int K, int num_sms, int cta, int* first, int* end);
 int bitdelta_gemm_plan_item_cta(int B, int m, int N, int K, int num_sms, int item);
 

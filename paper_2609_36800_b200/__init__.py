@@ -19,6 +19,7 @@ from .binding import (  # noqa: F401
     gemm_plan,
     gemm_plan_cta_items,
     gemm_plan_item_cta,
+    gemm_row_stream,
     gemm_workspace_bytes,
     kernel_launch_count,
     last_device_status,

@@ -24,7 +24,7 @@ EXPORTS = (
     "bitdelta_pack", "bitdelta_unpack", "bitdelta_compress_workspace_bytes", "bitdelta_compress",
     "bitdelta_gemm_workspace_bytes", "bitdelta_workspace_init",
     "bitdelta_gemm", "bitdelta_gemm_ex", "bitdelta_gemm_noalloc", "bitdelta_gemm_simt", "bitdelta_gemm_host_arena_bytes", "bitdelta_gemm_host",
-    "bitdelta_gemm_plan", "bitdelta_gemm_plan_cta_items", "bitdelta_gemm_plan_item_cta",
+    "bitdelta_gemm_plan", "bitdelta_gemm_row_stream", "bitdelta_gemm_plan_cta_items", "bitdelta_gemm_plan_item_cta",
     "bitdelta_last_device_status", "bitdelta_kernel_launch_count", "bitdelta_status_string", "bitdelta_selftest_timeout",
 )
 
@@ -66,6 +66,7 @@ def load_library():
     lib.bitdelta_gemm_host_arena_bytes.restype = sz
     lib.bitdelta_gemm_host.argtypes = [vp, vp, vp, vp, vp, ci, ci, ci, ci, vp, sz, vp]
     lib.bitdelta_gemm_plan.argtypes = [ci, ci, ci, ci, ci, ctypes.POINTER(ci)]
+    lib.bitdelta_gemm_row_stream.argtypes = [ci, ci, ci, ci, ci]
     lib.bitdelta_gemm_plan_cta_items.argtypes = [ci, ci, ci, ci, ci, ci, ctypes.POINTER(ci), ctypes.POINTER(ci)]
     lib.bitdelta_gemm_plan_item_cta.argtypes = [ci, ci, ci, ci, ci, ci]
     lib.bitdelta_last_device_status.argtypes = [vp, ctypes.POINTER(ci)]
@@ -237,6 +238,11 @@ def gemm_plan(B: int, m: int, N: int, K: int, num_sms: int = 148) -> dict:
     info = (ctypes.c_int * 16)()
     _check(load_library().bitdelta_gemm_plan(B, m, N, K, num_sms, info), "bitdelta_gemm_plan")
     return dict(zip(PLAN_FIELDS, list(info)))
+
+
+def gemm_row_stream(B: int, m: int, N: int, K: int, num_sms: int = 148) -> bool:
+    """Whether bitdelta_gemm runs this shape on the row-stream kernel (gemm_plan then reports what that stands in for)."""
+    return bool(load_library().bitdelta_gemm_row_stream(B, m, N, K, num_sms))
 
 
 def gemm_plan_cta_items(B: int, m: int, N: int, K: int, cta: int, num_sms: int = 148):

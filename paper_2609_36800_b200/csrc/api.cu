@@ -11,6 +11,7 @@
 #include <mutex>
 
 #include "../../include/bitdelta.h"
+#include "gemm_row.h"
 #include "gemm_tc.h"
 #include "plan.h"
 
@@ -102,12 +103,12 @@ int check_gemm_args(const void* X, const void* W, const void* bits, const void* 
 // row each, swizzled) x box_rows, i.e. a whole 128-k stage tile in ONE bulk-tensor operation, landing in
 // shared memory atom after atom.  (The number of bulk operations a CTA keeps in flight is what limits
 // its load throughput, not their size.)  Coordinates: (0, first row, k / 64).
-bool encode_bf16_tile(CUtensorMap* map, const void* ptr, uint64_t rows, uint64_t K, uint32_t box_rows) {
+bool encode_bf16_tile(CUtensorMap* map, const void* ptr, uint64_t rows, uint64_t K, uint32_t box_rows, uint32_t atoms = 2) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
     cuuint64_t dims[3] = {64, rows, K / 128 * 2};   // (whole 128-k steps)
     cuuint64_t strides[2] = {K * 2, 128};
-    cuuint32_t box[3] = {64, box_rows, 2};
+    cuuint32_t box[3] = {64, box_rows, atoms};
     cuuint32_t estr[3] = {1, 1, 1};
     return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -143,15 +144,16 @@ bool encode_u8_2d(CUtensorMap* map, const void* ptr, uint64_t rows, uint64_t K, 
 
 // 3-D uint32 [B, N, K/32], box = `box_words` words (8: the signs of 256 k, 32 bytes; 4: of 128 k) x 128 rows x tenants.
 bool encode_bits_3d(CUtensorMap* map, const void* ptr, uint64_t B, uint64_t N, uint64_t words, uint32_t tenants,
-                    uint32_t box_words = 8) {
+                    uint32_t box_words = 8, uint32_t box_rows = 128) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
     cuuint64_t dims[3] = {words, N, B};
     cuuint64_t strides[2] = {words * 4, words * 4 * N};
-    cuuint32_t box[3] = {box_words, 128, tenants};
+    cuuint32_t box[3] = {box_words, box_rows, tenants};   // (32 words = 128 bytes: swizzled, the rows are read by lanes)
     cuuint32_t estr[3] = {1, 1, 1};
     return fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT32, 3, const_cast<void*>(ptr), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, box_words == 32 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
+              CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -179,6 +181,18 @@ int whole_override() {
 bool early_start_enabled() {
     const char* e = getenv("BITDELTA_EARLY_START");   // (read at every call: bench.py times both settings in one process)
     return !(e && e[0] == '0');
+}
+
+// The row-stream decode kernel: by default where it pays (row_plan.h); BITDELTA_ROW=1: wherever it applies, =0: never.  A choice
+// of the other decode kernels (BITDELTA_FP4 and its variants, BITDELTA_CLUSTER) leaves the call to them.
+bool take_row_kernel(int B, int m, int N, int K, int sms) {
+    const char* e = getenv("BITDELTA_ROW");
+    if (e && e[0] == '0') return false;
+    const bd::RowPlan p = bd::make_row_plan(B, m, N, K, sms);
+    if (e && e[0] == '1') return p.ok;
+    if (!bd::row_kernel_pays(p, B, N, K)) return false;
+    return bd::fp4_mode() == 2 && bd::cluster_enabled() && !getenv("BITDELTA_FP4_INKERNEL") && !getenv("BITDELTA_FP4_RESIDENT") &&
+           !getenv("BITDELTA_FP4_COOP");
 }
 
 // Encoded tensor maps, kept per (kind, pointer, shape, box): encoding one costs a microsecond or two of host time,
@@ -354,6 +368,27 @@ int bitdelta_gemm_ex(const void* X, const void* W_base, const uint32_t* bits, co
 
     const bool plain = !f16 && act == BITDELTA_ACT_NONE && bias == nullptr;   // (the 4-bit decode kernel takes no options)
     bd::Plan p = bd::make_plan(B, m, N, K, d.sms, tb_override(), whole_override(), true, wide, plain);
+    if (!wide && p.ok && workspace && workspace_bytes >= p.ws_bytes && aligned16(workspace) && take_row_kernel(B, m, N, K, d.sms)) {
+        // (the row-stream kernel needs no scratch; a call that is refused for its workspace stays refused)
+        const bd::RowPlan rp = bd::make_row_plan(B, m, N, K, d.sms);
+        CUtensorMap rW, rX, rB;
+        if (!cached_map(&rW, MapKey{4, W_base, (uint64_t)N, (uint64_t)K, 0, (uint32_t)rp.rows, 16u},
+                        [&](CUtensorMap* mp) { return encode_bf16_tile(mp, W_base, (uint64_t)N, (uint64_t)K, (uint32_t)rp.rows, 16u); }) ||
+            !cached_map(&rX, MapKey{4, X, (uint64_t)B * m, (uint64_t)K, 0, 8u, 16u},
+                        [&](CUtensorMap* mp) { return encode_bf16_tile(mp, X, (uint64_t)B * m, (uint64_t)K, 8u, 16u); }) ||
+            !cached_map(&rB, MapKey{5, bits, (uint64_t)B, (uint64_t)N, (uint64_t)(K / 32), (uint32_t)rp.TB, (uint32_t)rp.rows},
+                        [&](CUtensorMap* mp) { return encode_bits_3d(mp, bits, (uint64_t)B, (uint64_t)N, (uint64_t)(K / 32), (uint32_t)rp.TB, 32u, (uint32_t)rp.rows); }))
+            return BITDELTA_ERR_CUDA;
+        bd::RowArgs ra{};
+        ra.B = B; ra.m = m; ra.N = N; ra.K = K; ra.f16 = f16; ra.act = act;
+        ra.TB = rp.TB; ra.rows = rp.rows; ra.groups = rp.groups; ra.units = rp.units; ra.stages = rp.stages; ra.k_stages = rp.k_stages;
+        ra.s_off = rp.s_off; ra.x_off = rp.x_off; ra.stage_bytes = rp.stage_bytes;
+        ra.X = X; ra.W = W_base; ra.bias = bias; ra.bits = bits; ra.alpha = alpha; ra.Y = Y;
+        const bool early = early_start_enabled() && g_weights_just_written.exchange(0) == 0;
+        if (bd::launch_gemm_row(rW, rX, rB, ra, rp, early, stream) != cudaSuccess) return BITDELTA_ERR_CUDA;
+        g_launches++;
+        return BITDELTA_OK;
+    }
     if (p.ok && p.pair) {
         // The pair schedule wants every pair resident at once (a cluster of two needs two free SMs of one
         // cluster-capable group); where the device cannot do that, run the one-CTA schedule.  Asked once per device.
@@ -522,6 +557,11 @@ int bitdelta_gemm_plan(int B, int m, int N, int K, int num_sms, int* info) {
     info[6] = p.teams; info[7] = (int)p.smem_bytes; info[8] = p.n_w; info[9] = p.n_x; info[10] = p.n_x8;
     info[11] = p.a_slots; info[12] = p.halves; info[13] = p.tok_tile; info[14] = p.groups; info[15] = p.n_tiles;
     return BITDELTA_OK;
+}
+
+int bitdelta_gemm_row_stream(int B, int m, int N, int K, int num_sms) {
+    if (B <= 0 || m <= 0 || N <= 0 || K <= 0 || (K % 32) != 0 || num_sms <= 0) return 0;
+    return take_row_kernel(B, m, N, K, num_sms) ? 1 : 0;
 }
 
 int bitdelta_gemm_plan_cta_items(int B, int m, int N, int K, int num_sms, int cta, int* first, int* end) {

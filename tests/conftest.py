@@ -8,6 +8,13 @@ if ROOT not in sys.path:
     sys.path.insert(0, ROOT)
 
 
+@pytest.fixture(autouse=True)
+def tcgen05_decode_kernels(request, monkeypatch):
+    """The tests of the 4-bit decode kernel's default route take it also at the sizes that the row-stream kernel has."""
+    if request.module.__name__ == "test_gpu_fp4":
+        monkeypatch.setenv("BITDELTA_ROW", "0")
+
+
 def pytest_configure(config):
     config.addinivalue_line("markers", "gpu: needs a CUDA device (sm_100a)")
 
