@@ -101,10 +101,10 @@ static_assert(sizeof(FCtl) <= kSmemCtrlBytes, "control block too large");
 
 // Eight signs per register: register c, nibble i <- bit 4i + c of the word (1 -> +1.0 = 0x2, 0 -> -1.0 = 0xA).
 __device__ __forceinline__ void decode_word_e2m1(uint32_t w, uint32_t* r) {
-    r[0] = ((w << 3) & 0x88888888u) ^ 0xAAAAAAAAu;
-    r[1] = ((w << 2) & 0x88888888u) ^ 0xAAAAAAAAu;
-    r[2] = ((w << 1) & 0x88888888u) ^ 0xAAAAAAAAu;
-    r[3] = (w & 0x88888888u) ^ 0xAAAAAAAAu;
+    r[0] = and_xor(w << 3, 0x88888888u, 0xAAAAAAAAu);
+    r[1] = and_xor(w << 2, 0x88888888u, 0xAAAAAAAAu);
+    r[2] = and_xor(w << 1, 0x88888888u, 0xAAAAAAAAu);
+    r[3] = and_xor(w, 0x88888888u, 0xAAAAAAAAu);
 }
 
 // Eight 16-bit values hv[i] of one token row (k = k0 + 4i) -> for every digit q the register R[q] whose nibble i is

@@ -7,7 +7,7 @@
 // of a stage each and keep fp32 sums in registers; at the end of a unit the eight partial sums are added in shared memory.
 // There is no activation pre-pass, no tensor-memory hand-over, no workspace and no sum across blocks: for few tenants
 // those latencies are most of a call of the other decode kernels (1 x 8 x 1024 x 1024: 2.3 us, 5.6 there; 8 x 1 x 2048 x 2048:
-// 7.4 and 13.9; 1 x 1 x 4096 x 4096: 9.2 and 10.5, 4.1 TB/s).
+// 6.7 and 13.6; 1 x 1 x 4096 x 4096: 8.9 and 10.5, 4.0 TB/s).
 //
 // The products run on mma.sync (m16n8k16, the weights on the 16-row side), because its A operand comes from registers, where the
 // decoded signs are; that path is a quarter as fast as tcgen05, which is what limits the kernel to few tenants.
@@ -75,10 +75,19 @@ template <bool kF16> __host__ __device__ constexpr uint32_t row_mid(int c) {
                                : (c == 7 ? 0x4040u : c == 6 ? 0x40A0u : c == 5 ? 0x4110u : 0x4188u));
 }
 // (`cst`: the four constants, class c at index c & 3; in registers, for the one logic operation takes only one immediate)
-template <bool kF16> __device__ __forceinline__ uint32_t row_sign_pair(uint32_t w, int p, const uint32_t (&cst)[4]) {   // (p: a constant after unrolling)
-    const int c = row_class<kF16>(p), s = row_shift<kF16>(p);
-    const uint32_t v = s > 0 ? w << s : w >> -s;
-    return (v & (0x00010001u << c)) | cst[c & 3];
+template <bool kF16> __device__ __forceinline__ uint32_t row_sign_pair(uint32_t v, int p, const uint32_t (&cst)[4]) {   // (p: a constant after unrolling)
+    const int c = row_class<kF16>(p);
+    uint32_t d;   // (one operation, written out: 8 x 1 x 4096 x 4096 17.4 us, 20.3 with the compiler's two)
+    asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(d) : "r"(v), "r"(0x00010001u << c), "r"(cst[c & 3]));   // (v & mask) | constant
+    return d;
+}
+// The word shifted for position p and its neighbours with the same shift (opaque: the compiler would otherwise fold the
+// shift into every logic operation's mask and shift each result).
+template <bool kF16> __device__ __forceinline__ uint32_t row_shifted(uint32_t w, int p) {
+    const int s = row_shift<kF16>(p);
+    uint32_t v = s > 0 ? w << s : w >> -s;
+    asm("" : "+r"(v));
+    return v;
 }
 
 // kTpt: tenants per activation tile, kNt: activation tiles per unit.
@@ -195,7 +204,7 @@ bitdelta_gemm_row_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
                     for (int q = 0; q < 4; ++q)
                         x[q] = lds128(st + a.x_off + i * 16384u + xrow * 128u + (uint32_t)(((c0 + (q ^ flip)) ^ (xrow & 7)) << 4));
                     // the tenants' sign words of the rows g, g + 8 (tenants past the unit's own: the first one's, not used)
-                    uint32_t sw[kTpt][2];
+                    uint32_t sw[kTpt][2], sv[kTpt][2];
 #pragma unroll
                     for (int j = 0; j < kTpt; ++j) {
                         const int jj = i * kTpt + j < nten ? i * kTpt + j : 0;
@@ -236,9 +245,19 @@ bitdelta_gemm_row_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
                             mma16816<kF16>(Z[i], o0, o0, o1, o1, xp[2 * q], xp[2 * q + 1]);
                         }
 #pragma unroll
-                        for (int j = 0; j < kTpt; ++j)
-                            mma16816<kF16>(accd[i][j], row_sign_pair<kF16>(sw[j][0], 2 * q, cst), row_sign_pair<kF16>(sw[j][1], 2 * q, cst),
-                                           row_sign_pair<kF16>(sw[j][0], 2 * q + 1, cst), row_sign_pair<kF16>(sw[j][1], 2 * q + 1, cst), xp[2 * q], xp[2 * q + 1]);
+                        for (int j = 0; j < kTpt; ++j) {
+                            if (q == 0 || row_shift<kF16>(2 * q) != row_shift<kF16>(2 * q - 1)) {
+                                sv[j][0] = row_shifted<kF16>(sw[j][0], 2 * q);
+                                sv[j][1] = row_shifted<kF16>(sw[j][1], 2 * q);
+                            }
+                            const uint32_t a0 = row_sign_pair<kF16>(sv[j][0], 2 * q, cst), a1 = row_sign_pair<kF16>(sv[j][1], 2 * q, cst);
+                            if (row_shift<kF16>(2 * q + 1) != row_shift<kF16>(2 * q)) {
+                                sv[j][0] = row_shifted<kF16>(sw[j][0], 2 * q + 1);
+                                sv[j][1] = row_shifted<kF16>(sw[j][1], 2 * q + 1);
+                            }
+                            mma16816<kF16>(accd[i][j], a0, a1, row_sign_pair<kF16>(sv[j][0], 2 * q + 1, cst), row_sign_pair<kF16>(sv[j][1], 2 * q + 1, cst),
+                                           xp[2 * q], xp[2 * q + 1]);
+                        }
                     }
                 }
             };

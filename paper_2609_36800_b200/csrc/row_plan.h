@@ -61,10 +61,10 @@ inline RowPlan make_row_plan(int B, int m, int N, int K, int num_sms) {
 }
 
 // Where the row-stream kernel is taken by default: one or two tenants, or up to 48 M signs including the tenant columns computed
-// for nothing.  Its MMAs cost ~1.5 us per tenant at 4096 x 4096, the others' latencies are the same whatever the size.
-// Measured (us, row-stream / the others): 1 x 1 x 4096 x 4096 9.2 / 10.5, 1 x 8 x 4096 x 11008 17.2 / 22.9, 2 x 1 x 4096 x 4096
-// 11.5 / 11.6, 2 x 8 11.6 / 13.7, 8 x 1 x 2048 x 2048 7.4 / 13.9, 8 x 8 x 1024 x 1024 4.2 / 12.4, 4 x 2 x 5632 x 2048 11.1 / 18.3,
-// 16 x 1 x 2048 x 768 6.3 / 14.9; beyond: 3 x 1 x 4096 x 4096 14.6 / 11.7, 8 x 1 20.2 / 14.8, 28 x 1 x 6400 x 816 28.3 / 21.2.
+// for nothing.  Its MMAs cost ~1.2 us per tenant at 4096 x 4096, the others' latencies are the same whatever the size.
+// Measured (us, row-stream / the others): 1 x 1 x 4096 x 4096 8.9 / 10.5, 1 x 8 x 4096 x 11008 17.2 / 22.9, 2 x 1 x 4096 x 4096
+// 10.5 / 10.9, 2 x 8 11.6 / 13.7, 8 x 1 x 2048 x 2048 6.7 / 13.6, 8 x 8 x 1024 x 1024 4.2 / 12.4, 4 x 2 x 5632 x 2048 11.1 / 18.3,
+// 16 x 1 x 2048 x 768 6.3 / 14.9; beyond: 4 x 1 x 4096 x 4096 12.9 / 11.9, 8 x 1 17.4 / 14.9, 28 x 1 x 6400 x 816 28.3 / 21.2.
 // (In the other direction a few are left to the others that it would win: 32 x 1 x 2048 x 1024 11.8 / 16.9.)
 inline bool row_kernel_pays(const RowPlan& p, int B, int N, int K) {
     return p.ok && (B <= 2 || (long long)p.tpt * p.nt * p.groups * N * K <= 48000000ll);
