@@ -7,7 +7,7 @@
 // of a stage each and keep fp32 sums in registers; at the end of a unit the eight partial sums are added in shared memory.
 // There is no activation pre-pass, no tensor-memory hand-over, no workspace and no sum across blocks: for few tenants
 // those latencies are most of a call of the other decode kernels (1 x 8 x 1024 x 1024: 2.3 us, 5.6 there; 8 x 1 x 2048 x 2048:
-// 6.7 and 13.6; 1 x 1 x 4096 x 4096: 8.9 and 10.5, 4.0 TB/s).
+// 6.7 and 13.6; 1 x 1 x 4096 x 4096: 8.7 and 10.5, 4.1 TB/s).
 //
 // The products run on mma.sync (m16n8k16, the weights on the 16-row side), because its A operand comes from registers, where the
 // decoded signs are; that path is a quarter as fast as tcgen05, which is what limits the kernel to few tenants.
@@ -100,8 +100,9 @@ bitdelta_gemm_row_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
     const uint32_t base = (raw + 1023u) & ~1023u;
     uint8_t* smem = smem_raw + (base - raw);
     const uint32_t red_off = (uint32_t)a.stages * a.stage_bytes;
-    float* red = reinterpret_cast<float*>(smem + red_off);                       // [warp][tile][column][16 rows]
-    RowCtl* ctl = reinterpret_cast<RowCtl*>(smem + red_off + kNt * kRowWarps * 128 * 4);
+    constexpr int kRedBufs = kNt < 4 ? 2 : 1;
+    constexpr int kRedFloats = kNt * kRowWarps * 128;                            // [warp][tile][column][16 rows]
+    RowCtl* ctl = reinterpret_cast<RowCtl*>(smem + red_off + kRedBufs * kRedFloats * 4);
     volatile uint32_t* abort_flag = &ctl->abort_flag;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -174,7 +175,11 @@ bitdelta_gemm_row_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
         for (int c = 0; c < 4; ++c) asm volatile("" : "+r"(cst[c]));
         const int m = a.m;
         const int jc[2] = {2 * t / m, (2 * t + 1) / m};   // the tenant of the tile that this thread's two columns belong to
-        for (int unit = (int)blockIdx.x; unit < a.units; unit += (int)gridDim.x) {
+        // The partial results of successive units go to two buffers in turn: a warp that writes a buffer again has passed the
+        // barrier of the unit between, which the others reach only after they have read it, so one barrier a unit is enough
+        // (2 x 1 x 4096 x 4096 10.5 -> 9.9 us, 2 x 4 x 1024 x 8192 8.4 -> 7.8).  Four activation tiles leave no room for two.
+        for (int unit = (int)blockIdx.x, odd = 0; unit < a.units; unit += (int)gridDim.x, odd ^= 1) {
+            float* red = reinterpret_cast<float*>(smem + red_off) + (kRedBufs == 2 ? odd * kRedFloats : 0);
             const int tile = unit / a.groups, grp = unit - tile * a.groups;
             const int n0 = tile * a.rows, tenant0 = grp * kTpt * kNt;
             const int nten = min(kTpt * kNt, a.B - tenant0);
@@ -318,7 +323,7 @@ bitdelta_gemm_row_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
                     }
                 }
             }
-            named_bar_sync(1, kRowWarps * 32);   // the partial sums are read: the next unit's may come
+            if constexpr (kRedBufs == 1) named_bar_sync(1, kRowWarps * 32);   // the partial sums are read: the next unit's may come
         }
     }
     __syncthreads();

@@ -49,7 +49,7 @@ inline RowPlan make_row_plan(int B, int m, int N, int K, int num_sms) {
     p.s_off = (uint32_t)p.rows * 128u * 16u;
     p.x_off = p.s_off + (uint32_t)round_up(p.TB * p.rows * 128, 1024);
     p.stage_bytes = p.x_off + (uint32_t)p.nt * 16384u;
-    const int red = p.nt * 8 * 128 * 4 + 1024;                    // the warps' partial results; barriers
+    const int red = (p.nt < 4 ? 2 : 1) * p.nt * 8 * 128 * 4 + 1024;   // the warps' partial results (of two units in turn); barriers
     int st = (kSmemBudget - 1024 - red) / (int)p.stage_bytes;
     if (st > kRowMaxStages) st = kRowMaxStages;
     if (st < 2) return p;
@@ -62,8 +62,8 @@ inline RowPlan make_row_plan(int B, int m, int N, int K, int num_sms) {
 
 // Where the row-stream kernel is taken by default: one or two tenants, or up to 48 M signs including the tenant columns computed
 // for nothing.  Its MMAs cost ~1.2 us per tenant at 4096 x 4096, the others' latencies are the same whatever the size.
-// Measured (us, row-stream / the others): 1 x 1 x 4096 x 4096 8.9 / 10.5, 1 x 8 x 4096 x 11008 17.2 / 22.9, 2 x 1 x 4096 x 4096
-// 10.5 / 10.9, 2 x 8 11.6 / 13.7, 8 x 1 x 2048 x 2048 6.7 / 13.6, 8 x 8 x 1024 x 1024 4.2 / 12.4, 4 x 2 x 5632 x 2048 11.1 / 18.3,
+// Measured (us, row-stream / the others): 1 x 1 x 4096 x 4096 8.7 / 10.5, 1 x 8 x 4096 x 11008 17.2 / 22.9, 2 x 1 x 4096 x 4096
+// 9.9 / 10.9, 2 x 8 11.3 / 13.5, 8 x 1 x 2048 x 2048 6.7 / 13.6, 8 x 8 x 1024 x 1024 4.2 / 12.4, 4 x 2 x 5632 x 2048 11.1 / 18.3,
 // 16 x 1 x 2048 x 768 6.3 / 14.9; beyond: 4 x 1 x 4096 x 4096 12.9 / 11.9, 8 x 1 17.4 / 14.9, 28 x 1 x 6400 x 816 28.3 / 21.2.
 // (In the other direction a few are left to the others that it would win: 32 x 1 x 2048 x 1024 11.8 / 16.9.)
 inline bool row_kernel_pays(const RowPlan& p, int B, int N, int K) {

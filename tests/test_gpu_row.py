@@ -114,7 +114,7 @@ def test_large_small_and_non_finite_activations(monkeypatch):
     fin = [(0, 0), (0, 1), (0, 2), (0, 3), (1, 1), (1, 3)]
     for b, t in fin:
         # one output rounding (2^-9) and the sums' 2^-20 of the largest magnitude that enters them
-        scale = np.abs(ref[b, t]) * 2.0**-8 + np.abs(x[b, t]).max() * K * 2.0**-20
+        scale = np.abs(ref[b, t]) * 2.0**-8 + np.abs(x[b, t].astype(np.float64)).max() * K * 2.0**-20
         assert (np.abs(got[b, t] - ref[b, t]) <= scale + 1e-30).all(), (b, t)
 
 
