@@ -233,8 +233,9 @@ int bitdelta_gemm_host(const void* X_host, const void* W_base_host, const uint32
  * is one 128-row tile of W_base for one group of TB tenants (decode schedules) or one tenant's token tile
  * (tiled schedule), a k-step is 128 k; item = unit * P + k-step.
  *
- * bitdelta_gemm_row_stream returns 1 for the shapes (few tenants, or small; m <= 8) that run on the row-stream kernel instead: one
- * launch, no scratch, a block per few weight rows with all of K.  bitdelta_gemm_plan reports the schedule that it stands
+ * bitdelta_gemm_row_stream returns 1 for the shapes (few tenants, or small; m <= 8; calls with options: a somewhat
+ * wider range) that run on the row-stream kernel instead: one launch, no scratch, a block per few weight rows with all
+ * of K.  bitdelta_gemm_plan reports the schedule that it stands
  * in for, which the same call takes with BITDELTA_ROW=0 in the environment.
  *
  * bitdelta_gemm_plan fills info[0 .. BITDELTA_PLAN_INFO_INTS-1] (host pointer):

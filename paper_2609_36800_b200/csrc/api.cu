@@ -185,12 +185,12 @@ bool early_start_enabled() {
 
 // The row-stream decode kernel: by default where it pays (row_plan.h); BITDELTA_ROW=1: wherever it applies, =0: never.  A choice
 // of the other decode kernels (BITDELTA_FP4 and its variants, BITDELTA_CLUSTER) leaves the call to them.
-bool take_row_kernel(int B, int m, int N, int K, int sms) {
+bool take_row_kernel(int B, int m, int N, int K, int sms, bool plain, int cluster) {
     const char* e = getenv("BITDELTA_ROW");
     if (e && e[0] == '0') return false;
     const bd::RowPlan p = bd::make_row_plan(B, m, N, K, sms);
     if (e && e[0] == '1') return p.ok;
-    if (!bd::row_kernel_pays(p, B, N, K)) return false;
+    if (!bd::row_kernel_pays(p, B, N, K, plain, cluster)) return false;
     return bd::fp4_mode() == 2 && bd::cluster_enabled() && !getenv("BITDELTA_FP4_INKERNEL") && !getenv("BITDELTA_FP4_RESIDENT") &&
            !getenv("BITDELTA_FP4_COOP");
 }
@@ -368,7 +368,7 @@ int bitdelta_gemm_ex(const void* X, const void* W_base, const uint32_t* bits, co
 
     const bool plain = !f16 && act == BITDELTA_ACT_NONE && bias == nullptr;   // (the 4-bit decode kernel takes no options)
     bd::Plan p = bd::make_plan(B, m, N, K, d.sms, tb_override(), whole_override(), true, wide, plain);
-    if (!wide && p.ok && workspace && workspace_bytes >= p.ws_bytes && aligned16(workspace) && take_row_kernel(B, m, N, K, d.sms)) {
+    if (!wide && p.ok && workspace && workspace_bytes >= p.ws_bytes && aligned16(workspace) && take_row_kernel(B, m, N, K, d.sms, plain, p.cluster)) {
         // (the row-stream kernel needs no scratch; a call that is refused for its workspace stays refused)
         const bd::RowPlan rp = bd::make_row_plan(B, m, N, K, d.sms);
         CUtensorMap rW, rX, rB;
@@ -561,7 +561,8 @@ int bitdelta_gemm_plan(int B, int m, int N, int K, int num_sms, int* info) {
 
 int bitdelta_gemm_row_stream(int B, int m, int N, int K, int num_sms) {
     if (B <= 0 || m <= 0 || N <= 0 || K <= 0 || (K % 32) != 0 || num_sms <= 0) return 0;
-    return take_row_kernel(B, m, N, K, num_sms) ? 1 : 0;
+    const bd::Plan p = bd::make_plan(B, m, N, K, num_sms, tb_override(), whole_override());
+    return p.ok && take_row_kernel(B, m, N, K, num_sms, true, p.cluster) ? 1 : 0;
 }
 
 int bitdelta_gemm_plan_cta_items(int B, int m, int N, int K, int num_sms, int cta, int* first, int* end) {

@@ -66,8 +66,12 @@ inline RowPlan make_row_plan(int B, int m, int N, int K, int num_sms) {
 // 9.9 / 10.9, 2 x 8 11.3 / 13.5, 8 x 1 x 2048 x 2048 6.7 / 13.6, 8 x 8 x 1024 x 1024 4.2 / 12.4, 4 x 2 x 5632 x 2048 11.1 / 18.3,
 // 16 x 1 x 2048 x 768 6.3 / 14.9; beyond: 4 x 1 x 4096 x 4096 12.9 / 11.9, 8 x 1 17.4 / 14.9, 28 x 1 x 6400 x 816 28.3 / 21.2.
 // (In the other direction a few are left to the others that it would win: 32 x 1 x 2048 x 1024 11.8 / 16.9.)
-inline bool row_kernel_pays(const RowPlan& p, int B, int N, int K) {
-    return p.ok && (B <= 2 || (long long)p.tpt * p.nt * p.groups * N * K <= 48000000ll);
+// Calls with options or binary16 operands have the slower 8-bit kernel as the alternative: up to 68 M (4 x 1 x 4096 x 4096
+// binary16 12.3 / 14.8, 4 x 8 17.5 / 20.5; beyond, 8 x 1 x 1024 x 8448 with a gate 14.2 / 13.3).  Where the 4-bit kernel's clusters of two or four blocks apply (`cluster`), it is ahead
+// from 32 M on (3 x 1 x 2048 x 4096 8.5 / 7.9, 4 x 1 x 2816 x 4096 10.2 / 9.5; without clusters 8 x 1 x 2048 x 2816 10.2 / 14.4).
+inline bool row_kernel_pays(const RowPlan& p, int B, int N, int K, bool plain, int cluster) {
+    const long long limit = !plain ? 68000000ll : (cluster == 2 || cluster == 4) ? 32000000ll : 48000000ll;
+    return p.ok && (B <= 2 || (long long)p.tpt * p.nt * p.groups * N * K <= limit);
 }
 
 }  // namespace bd
