@@ -198,7 +198,7 @@ inline Plan make_plan(int B, int m, int N, int K, int num_sms, int tb_override =
         // 128; a tenant's tokens are spread evenly over its tiles.  The tiles' loads from L2 weigh on the schedule (31 bytes per
         // cycle and multiprocessor at 128 tokens), and a half-empty last tile costs as much as a full one: 4 x 512 x 4096 x
         // 4096 in tiles of 128: 103.5 us, of 176: 97.7; 4 x 130: 53.4 (two of 128) and 34.5 (one of 144); 2 x 300 x 4096 x
-        // 11008 binary16 with a gate: 115.9 (three of 128) and 97.6 (two of 160).
+        // 11008 binary16 with a gate: 115.9 (three of 128) and 95.9 (two of 160).
         const bool pairs = allow_pair && pair_enabled() && m > 64 && (p.n_tiles % 2) == 0 && num_sms >= 2;
         p.m_tiles = (m + (pairs ? kMaxTokTile : 128) - 1) / (pairs ? kMaxTokTile : 128);
         p.tok_tile = round_up((m + p.m_tiles - 1) / p.m_tiles, 16);
