@@ -81,7 +81,7 @@ struct Plan {
     uint32_t w_stage_bytes, x_tile_bytes, w_atom_bytes, x_atom_bytes, x8_atom_bytes, bslot_bytes, smem_bytes;
     uint32_t col_base, col_delta, col_a;
     size_t slot_floats;   // floats of one partial-result slot: 128 rows x tokens per unit
-    size_t ws_header_bytes;   // arrival counters: one u32 per work unit
+    size_t ws_header_bytes;   // arrival counters: one u32 per work unit (the same size in all plans of a shape)
     size_t ws_partials_bytes; // two partial-result slots per CTA
     size_t ws_x8_bytes;       // decode: e5m2 pieces of X, [B, 4, m, K] bytes
     size_t ws_bytes;
@@ -117,6 +117,18 @@ inline bool fp4_bits16_enabled() {
 inline bool cluster_enabled() {
     const char* e = getenv("BITDELTA_CLUSTER");
     return !(e && e[0] == '0');
+}
+
+// The largest number of groups among the plans of one shape (see the workspace header).
+inline int header_groups(const Plan& p, int B, int m, int K) {
+    int g = 1;
+    if (m <= kDecodeMaxM && (K % kPairK) == 0) {
+        g = (B + (m <= 4 ? 8 : 4) - 1) / (m <= 4 ? 8 : 4);      // (decode; the wide-range plan takes at least as many tenants a unit)
+    } else if (m > 64 || B == 1) {
+        const int tile = round_up((m + (m + 127) / 128 - 1) / ((m + 127) / 128), 16);   // (tiles of 128: what a device without room for the pairs takes)
+        g = B * ((m + tile - 1) / tile);
+    }
+    return g > p.groups ? g : p.groups;
 }
 
 // allow_pair = false: the device cannot hold all the pairs (or clusters) at once (see the launcher), plan without them.
@@ -435,8 +447,11 @@ inline Plan make_plan(int B, int m, int N, int K, int num_sms, int tb_override =
 
     // Workspace: arrival counters, two partial-result slots per CTA, then (decode) the e5m2
     // pieces of X written by the activation-split kernel.
-    p.ws_header_bytes = (size_t)round_up((p.n_tiles * p.groups + 1) * 4, 1024);   // one arrival counter per W_base tile and group,
-                                                                                  // and (last word) the activation-image counter of the 4-bit kernel
+    // One arrival counter per W_base tile and group, and (last word) the activation-image counter of the 4-bit kernel.  Room for
+    // the plan with the most groups that a call of this shape can take (decode or wide range, on pairs or not): the calls may
+    // share a workspace, and the counters of one must not lie in the partial results of another.
+    const int groups_max = header_groups(p, B, m, K);
+    p.ws_header_bytes = (size_t)round_up((p.n_tiles * groups_max + 1) * 4, 1024);
     // (sized for the largest grid any device could get, so that the size does not depend on the device;
     // never more CTAs than items)
     const long long items = p.pair ? 2 * p.T : p.T;
