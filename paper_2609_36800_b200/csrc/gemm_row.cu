@@ -267,7 +267,8 @@ bitdelta_gemm_row_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
                 }
             };
             for (int s = 0; s < a.k_stages; ++s) {
-                ok = ok && wait_bar(smem_u32(&ctl->full[slot]), phase, abort_flag, 41);
+                // (one answer per warp: its lanes leave the wait one by one, and the matrix instructions below need all of them)
+                ok = warp_all(ok && wait_bar(smem_u32(&ctl->full[slot]), phase, abort_flag, 41));
                 if (ok && s * kRowStageK + warp * 128 < a.K) {
                     if (new_z) stage(std::true_type{});
                     else stage(std::false_type{});
