@@ -7,7 +7,11 @@ back to the CPU: a missing library or a non-sm_100 device raises.
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
+
+from .build import fastcall_path
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 # BITDELTA_LIB points at another build of the same library (the trace build made by `build.py --trace`).
@@ -37,6 +41,22 @@ class BitDeltaError(RuntimeError):
 
 def library_path() -> str:
     return _LIB_PATH
+
+
+def _load_fastcall(gemm_ex: int):
+    """The extension module's `gemm`, calling bitdelta_gemm_ex at that address; None where none is built for this torch and
+    Python (its file name says which): every call then goes through the checks of `gemm` below."""
+    path = fastcall_path()
+    if path is None or not os.path.exists(path):
+        return None
+    loader = importlib.machinery.ExtensionFileLoader("_fastcall", path)
+    try:
+        module = importlib.util.module_from_spec(importlib.util.spec_from_loader("_fastcall", loader))
+        loader.exec_module(module)
+    except ImportError:
+        return None
+    module.set_library(gemm_ex)
+    return module.gemm
 
 
 def load_library():
@@ -77,13 +97,7 @@ def load_library():
     for fn in ("bitdelta_pack", "bitdelta_unpack", "bitdelta_compress", "bitdelta_workspace_init", "bitdelta_gemm",
                "bitdelta_gemm_simt", "bitdelta_gemm_noalloc", "bitdelta_gemm_host", "bitdelta_last_device_status"):
         getattr(lib, fn).restype = ci
-    try:
-        import torch   # noqa: F401  (the extension module links against its libraries)
-        from . import _fastcall
-        _fastcall.set_library(ctypes.cast(lib.bitdelta_gemm_ex, vp).value)
-        _fast = _fastcall.gemm
-    except ImportError:   # (not built against this torch: every call goes through the checks below)
-        _fast = None
+    _fast = _load_fastcall(ctypes.cast(lib.bitdelta_gemm_ex, vp).value)
     _lib = lib
     return lib
 

@@ -8,13 +8,13 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(CSRC, "build")
 LIB = os.path.join(HERE, "libbitdelta.so")
-FASTCALL = os.path.join(HERE, "_fastcall.so")   # CPython entry of the product (csrc/fastcall.cpp)
 SOURCES = ["api.cu", "gemm_tc.cu", "gemm_fp4.cu", "gemm_row.cu", "kernels_simple.cu"]
 HEADERS = ["ptx.cuh", "plan.h", "gemm_tc.h", "gemm_common.cuh", "gemm_row.h", "row_plan.h", os.path.join("..", "..", "include", "bitdelta.h")]
 ARCH = ["-gencode", "arch=compute_100a,code=sm_100a"]
@@ -29,24 +29,35 @@ def _newest_header() -> float:
     return max(os.path.getmtime(os.path.join(CSRC, h)) for h in HEADERS if os.path.exists(os.path.join(CSRC, h)))
 
 
-def build_fastcall(force: bool = False) -> str:
-    """csrc/fastcall.cpp as the extension module _fastcall, against the installed torch's headers (host code only)."""
-    src = os.path.join(CSRC, "fastcall.cpp")
-    if not force and os.path.exists(FASTCALL) and os.path.getmtime(FASTCALL) > os.path.getmtime(src):
-        return FASTCALL
-    import sysconfig
+def fastcall_path():
+    """The extension module of csrc/fastcall.cpp (the product's CPython entry), named after what it is built against: it reads
+    torch's tensors by their layout, so one of another torch or Python must not be loaded.  None without torch."""
+    try:
+        import torch
+    except ImportError:
+        return None
+    commit = (getattr(torch.version, "git_version", None) or "")[:8]
+    return os.path.join(HERE, f"_fastcall.torch-{torch.__version__}-{commit}{sysconfig.get_config_var('EXT_SUFFIX')}")
 
+
+def fastcall_is_stale() -> bool:
+    path = fastcall_path()
+    return path is not None and not (os.path.exists(path) and os.path.getmtime(path) > os.path.getmtime(os.path.join(CSRC, "fastcall.cpp")))
+
+
+def build_fastcall() -> None:
+    """csrc/fastcall.cpp against the installed torch's headers (host code only)."""
     import torch
     from torch.utils import cpp_extension
     inc = [*cpp_extension.include_paths(), sysconfig.get_paths()["include"], os.path.join(os.path.dirname(os.path.dirname(_nvcc())), "include")]
     libs = os.path.join(os.path.dirname(torch.__file__), "lib")
     subprocess.run(["g++", "-std=c++17", "-O2", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
-                    *(f"-I{d}" for d in inc), src, "-o", FASTCALL, f"-L{libs}", "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"], check=True)
-    return FASTCALL
+                    *(f"-I{d}" for d in inc), os.path.join(CSRC, "fastcall.cpp"), "-o", fastcall_path(), f"-L{libs}", "-ltorch_python",
+                    "-ltorch_cpu", "-lc10", "-lc10_cuda"], check=True)
 
 
 def is_stale() -> bool:
-    if not os.path.exists(LIB) or not os.path.exists(FASTCALL) or os.path.getmtime(os.path.join(CSRC, "fastcall.cpp")) > os.path.getmtime(FASTCALL):
+    if not os.path.exists(LIB):
         return True
     t = os.path.getmtime(LIB)
     deps = [os.path.join(CSRC, f) for f in SOURCES + HEADERS]
@@ -71,14 +82,16 @@ def _compile(src: str, force: bool, verbose: bool, trace: bool = False, steps: b
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    if not force and not is_stale():
-        return LIB
-    os.makedirs(OBJ, exist_ok=True)
+    library, fastcall = force or is_stale(), force or fastcall_is_stale()
     with ThreadPoolExecutor(max_workers=len(SOURCES) + 1) as pool:
-        fast = pool.submit(build_fastcall, force)
-        objs = list(pool.map(lambda s: _compile(s, force, verbose), SOURCES))
-        fast.result()
-    subprocess.run([_nvcc(), *ARCH, "-shared", "-cudart", "shared", "-o", LIB, *objs], check=True)
+        fast = pool.submit(build_fastcall) if fastcall else None
+        if library:
+            os.makedirs(OBJ, exist_ok=True)
+            objs = list(pool.map(lambda s: _compile(s, force, verbose), SOURCES))
+        if fast:
+            fast.result()
+    if library:
+        subprocess.run([_nvcc(), *ARCH, "-shared", "-cudart", "shared", "-o", LIB, *objs], check=True)
     return LIB
 
 

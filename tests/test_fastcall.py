@@ -65,3 +65,18 @@ def test_both_routes_give_the_same_result_and_the_same_refusals(dtype, bias, act
     slow = run()
     torch.cuda.synchronize()
     assert torch.equal(fast.view(torch.int16), slow.view(torch.int16)) and torch.equal(on_side.view(torch.int16), slow.view(torch.int16))
+
+
+def _child(code):
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    return subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True)
+
+
+@pytest.mark.parametrize("other", ["torch.__version__ = '2.0.0'", "import sysconfig; sysconfig._CONFIG_VARS['EXT_SUFFIX'] = '.cpython-39-x86_64-linux-gnu.so'"])
+def test_a_module_built_against_another_torch_or_python_is_not_loaded(other):
+    r = _child(f"import torch, sysconfig; sysconfig.get_config_vars(); {other}; import paper_2609_36800_b200 as bd; bd.load_library(); "
+               "assert bd.binding._fast is None")
+    assert r.returncode == 0, r.stderr
