@@ -82,16 +82,17 @@ def _compile(src: str, force: bool, verbose: bool, trace: bool = False, steps: b
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    library, fastcall = force or is_stale(), force or fastcall_is_stale()
-    with ThreadPoolExecutor(max_workers=len(SOURCES) + 1) as pool:
-        fast = pool.submit(build_fastcall) if fastcall else None
-        if library:
-            os.makedirs(OBJ, exist_ok=True)
+    if force or is_stale():
+        os.makedirs(OBJ, exist_ok=True)
+        with ThreadPoolExecutor(max_workers=len(SOURCES)) as pool:
             objs = list(pool.map(lambda s: _compile(s, force, verbose), SOURCES))
-        if fast:
-            fast.result()
-    if library:
         subprocess.run([_nvcc(), *ARCH, "-shared", "-cudart", "shared", "-o", LIB, *objs], check=True)
+    if force or fastcall_is_stale():
+        # (the library does not depend on it: without torch, its headers or g++ the product's calls go through the binding's checks)
+        try:
+            build_fastcall()
+        except (ImportError, OSError, subprocess.CalledProcessError) as e:
+            print(f"the product's native entry was not built ({e}); calls go through Python", file=sys.stderr)
     return LIB
 
 

@@ -80,3 +80,19 @@ def test_a_module_built_against_another_torch_or_python_is_not_loaded(other):
     r = _child(f"import torch, sysconfig; sysconfig.get_config_vars(); {other}; import paper_2609_36800_b200 as bd; bd.load_library(); "
                "assert bd.binding._fast is None")
     assert r.returncode == 0, r.stderr
+
+
+@pytest.mark.parametrize("error", ["ImportError('no torch')", "FileNotFoundError('g++')", "subprocess.CalledProcessError(1, 'g++')"])
+def test_the_library_is_built_without_the_module(error):
+    # (nothing is compiled or linked: the steps are replaced by records of them)
+    r = _child(f"""
+import subprocess
+from paper_2609_36800_b200 import build
+ran = []
+def fail(*a): raise {error}
+build.build_fastcall, build._compile = fail, lambda src, *a: src
+build.subprocess.run = lambda cmd, **kw: ran.append(cmd)
+assert build.build(force=True) == build.LIB
+assert any(build.LIB in cmd for cmd in ran), ran
+""")
+    assert r.returncode == 0, r.stderr
