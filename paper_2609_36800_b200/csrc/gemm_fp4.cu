@@ -100,9 +100,20 @@ struct FCtl {
 static_assert(sizeof(FCtl) <= kSmemCtrlBytes, "control block too large");
 
 // Eight signs per register: register c, nibble i <- bit 4i + c of the word (1 -> +1.0 = 0x2, 0 -> -1.0 = 0xA).
+// The cluster form takes the written-out operation (and_xor) for two registers of four only: with its few steps per block it is
+// not the integer rate that bounds it, and the faster decode runs into the copies of the next step.  Calls in a row on three sets of
+// operands (partly in L2), us with four / two / none of the registers: 8 x 1 x 4096 x 4096 15.85 / 15.53 / 15.63, 8 x 2 17.41 / 16.85 /
+// 16.95, 8 x 4 20.04 / 20.00 / 20.33; operands from DRAM, in a graph: 14.05 / 14.16 / 14.23, 15.50 / 15.57 / 15.71, 18.46 / 18.47 / 18.56.
+// The flat list takes it for all (16 x 4 x 4096 x 11008 52.9 -> 51.9).
+template <bool kCluster>
 __device__ __forceinline__ void decode_word_e2m1(uint32_t w, uint32_t* r) {
-    r[0] = and_xor(w << 3, 0x88888888u, 0xAAAAAAAAu);
-    r[1] = and_xor(w << 2, 0x88888888u, 0xAAAAAAAAu);
+    if constexpr (kCluster) {
+        r[0] = ((w << 3) & 0x88888888u) ^ 0xAAAAAAAAu;
+        r[1] = ((w << 2) & 0x88888888u) ^ 0xAAAAAAAAu;
+    } else {
+        r[0] = and_xor(w << 3, 0x88888888u, 0xAAAAAAAAu);
+        r[1] = and_xor(w << 2, 0x88888888u, 0xAAAAAAAAu);
+    }
     r[2] = and_xor(w << 1, 0x88888888u, 0xAAAAAAAAu);
     r[3] = and_xor(w, 0x88888888u, 0xAAAAAAAAu);
 }
@@ -845,16 +856,16 @@ bitdelta_gemm_fp4_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
                     if constexpr (kTB8) {
 #pragma unroll
                         for (int i = 0; i < 4; ++i) {
-                            decode_word_e2m1(s ? wq[i].z : wq[i].x, r + 8 * i);
-                            decode_word_e2m1(s ? wq[i].w : wq[i].y, r + 8 * i + 4);
+                            decode_word_e2m1<kForm == 1>(s ? wq[i].z : wq[i].x, r + 8 * i);
+                            decode_word_e2m1<kForm == 1>(s ? wq[i].w : wq[i].y, r + 8 * i + 4);
                         }
                     } else {
 #pragma unroll
                         for (int i = 0; i < 2; ++i) {
-                            decode_word_e2m1(wq[i].x, r + 16 * i);
-                            decode_word_e2m1(wq[i].y, r + 16 * i + 4);
-                            decode_word_e2m1(wq[i].z, r + 16 * i + 8);
-                            decode_word_e2m1(wq[i].w, r + 16 * i + 12);
+                            decode_word_e2m1<kForm == 1>(wq[i].x, r + 16 * i);
+                            decode_word_e2m1<kForm == 1>(wq[i].y, r + 16 * i + 4);
+                            decode_word_e2m1<kForm == 1>(wq[i].z, r + 16 * i + 8);
+                            decode_word_e2m1<kForm == 1>(wq[i].w, r + 16 * i + 12);
                         }
                     }
                     // (keeps the decode arithmetic above the waits: the compiler would otherwise sink it to the store)
