@@ -11,8 +11,6 @@ import importlib.machinery
 import importlib.util
 import os
 
-from .build import fastcall_path
-
 _HERE = os.path.dirname(os.path.abspath(__file__))
 # BITDELTA_LIB points at another build of the same library (the trace build made by `build.py --trace`).
 _LIB_PATH = os.environ.get("BITDELTA_LIB") or os.path.join(_HERE, "libbitdelta.so")
@@ -46,6 +44,7 @@ def library_path() -> str:
 def _load_fastcall(gemm_ex: int):
     """The extension module's `gemm`, calling bitdelta_gemm_ex at that address; None where none is built for this torch and
     Python (its file name says which): every call then goes through the checks of `gemm` below."""
+    from .build import fastcall_path
     path = fastcall_path()
     if path is None or not os.path.exists(path):
         return None
