@@ -383,7 +383,7 @@ int bitdelta_gemm_ex(const void* X, const void* W_base, const uint32_t* bits, co
         ra.B = B; ra.m = m; ra.N = N; ra.K = K; ra.f16 = f16; ra.act = act;
         ra.TB = rp.TB; ra.rows = rp.rows; ra.groups = rp.groups; ra.units = rp.units; ra.stages = rp.stages; ra.k_stages = rp.k_stages;
         ra.s_off = rp.s_off; ra.x_off = rp.x_off; ra.stage_bytes = rp.stage_bytes;
-        ra.X = X; ra.W = W_base; ra.bias = bias; ra.bits = bits; ra.alpha = alpha; ra.Y = Y;
+        ra.bias = bias; ra.alpha = alpha; ra.Y = Y;
         const bool early = early_start_enabled() && g_weights_just_written.exchange(0) == 0;
         if (bd::launch_gemm_row(rW, rX, rB, ra, rp, early, stream) != cudaSuccess) return BITDELTA_ERR_CUDA;
         g_launches++;

@@ -12,17 +12,14 @@
 // The products run on mma.sync (m16n8k16, the weights on the 16-row side), because its A operand comes from registers, where the
 // decoded signs are; that path is a quarter as fast as tcgen05, which is what limits the kernel to few tenants.
 //   * k is dealt to the threads of a fragment by words: thread t of a quad owns word t of the warp's 128 k, in both operands.
-//   * Signs cost ONE logic operation per two of them, and a shift per eight: bits p and p + 16 of a word (four classes of p after
-//     the shift) replace bit c of a pair of constants 2, 4, 8, 16, whose value then is o + s with o = 3, 5, 9, 17 and s = +-1.
-//     The constant part Z = sum_k o(k) x_k, the same for every weight row, comes from MMAs with the o(k) themselves and is
-//     subtracted at the end.  Magnitudes grow by about ten, i.e. three of fp32's 24 bits, in the delta term only; operands
-//     are exact.  An output that is not finite (infinities, NaN, sums beyond the range) is computed again term by term.
+//   * Signs are operands +-1, exactly: bits p and p + 16 of a word, shifted to the two halves' sign bits, flip the signs of a pair of
+//     ones (a shift and a logic operation per two of them).  Every product is exact, so the sums are as good as fp32 accumulation
+//     makes them, and infinities and NaN come out by themselves.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include <atomic>
-#include <type_traits>
 
 #include "gemm_common.cuh"
 #include "gemm_row.h"
@@ -32,6 +29,13 @@ namespace bd {
 
 constexpr int kRowWarps = 8;                                  // consumers; warp 8 is the producer
 constexpr int kRowThreads = (kRowWarps + 1) * 32;
+
+// The matrix unit truncates as it accumulates, so a long chain of MMAs drifts.  Up to kRowChainStages stages (eight MMAs per sum and
+// warp each) are one chain; a longer K is added up in chains of kRowLongStages, with rounded additions between them.  Error of the
+// delta's sum against 64 bits, relative, 2 x 8 x 14336 x 1024 in binary16 (the 8-bit kernel's beside it): N(0, 1) 1.7e-7 in one chain
+// (8.2e-7), heavy-tailed (N(0, 1) times exp(1.5 N(0, 1))) 1.5e-6 in one chain, 1.9e-7 in chains of two (1.8e-7).  Time: 1-2 % where
+// the chains are cut, which is why short K are not.
+constexpr int kRowChainStages = 4, kRowLongStages = 2;
 
 struct RowCtl {
     uint64_t full[kRowMaxStages], empty[kRowMaxStages];
@@ -60,38 +64,13 @@ __device__ __forceinline__ uint32_t lds32(uint32_t addr) {
     return v;
 }
 
-// Position p (0..15) of a sign word: the bit its two signs (p, p + 16) sit at after the shift, and the shift (left if positive).
-template <bool kF16> __host__ __device__ constexpr int row_class(int p) {
-    return kF16 ? (p < 3 ? p + 8 : p < 7 ? p + 4 : p < 11 ? p : p < 15 ? p - 4 : p - 8) : (p < 4 ? p + 4 : p < 8 ? p : p < 12 ? p - 4 : p - 8);
-}
-template <bool kF16> __host__ __device__ constexpr int row_shift(int p) { return row_class<kF16>(p) - p; }
-// The constants of a class: 2, 4, 8, 16 (bit c clear); with bit c set: + 2; the middle: 3, 5, 9, 17.
-template <bool kF16> __host__ __device__ constexpr uint32_t row_const(int c) {
-    return 0x00010001u * (kF16 ? (c == 10 ? 0x4000u : c == 9 ? 0x4400u : c == 8 ? 0x4800u : 0x4C00u)
-                               : (c == 7 ? 0x4000u : c == 6 ? 0x4080u : c == 5 ? 0x4100u : 0x4180u));
-}
-template <bool kF16> __host__ __device__ constexpr uint32_t row_mid(int c) {
-    return 0x00010001u * (kF16 ? (c == 10 ? 0x4200u : c == 9 ? 0x4500u : c == 8 ? 0x4880u : 0x4C40u)
-                               : (c == 7 ? 0x4040u : c == 6 ? 0x40A0u : c == 5 ? 0x4110u : 0x4188u));
-}
-// (`cst`: the four constants, class c at index c & 3; in registers, for the one logic operation takes only one immediate)
-template <bool kF16> __device__ __forceinline__ uint32_t row_sign_pair(uint32_t v, int p, const uint32_t (&cst)[4]) {   // (p: a constant after unrolling)
-    const int c = row_class<kF16>(p);
-    uint32_t d;   // (one operation, written out: 8 x 1 x 4096 x 4096 17.4 us, 20.3 with the compiler's two)
-    asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(d) : "r"(v), "r"(0x00010001u << c), "r"(cst[c & 3]));   // (v & mask) | constant
-    return d;
-}
-// The word shifted for position p and its neighbours with the same shift (opaque: the compiler would otherwise fold the
-// shift into every logic operation's mask and shift each result).
-template <bool kF16> __device__ __forceinline__ uint32_t row_shifted(uint32_t w, int p) {
-    const int s = row_shift<kF16>(p);
-    uint32_t v = s > 0 ? w << s : w >> -s;
-    asm("" : "+r"(v));
-    return v;
+// Signs p and p + 16 of a word as a pair of +-1 in the I/O type (`minus_one2`: two of -1, in a register: and_xor).
+__device__ __forceinline__ uint32_t row_sign_pair(uint32_t w, int p, uint32_t minus_one2) {   // (p: a constant after unrolling)
+    return and_xor(w << (15 - p), 0x80008000u, minus_one2);
 }
 
-// kTpt: tenants per activation tile, kNt: activation tiles per unit.
-template <bool kF16, int kTpt, int kNt>
+// kTpt: tenants per activation tile, kNt: activation tiles per unit, kLong: K beyond one chain.
+template <bool kF16, int kTpt, int kNt, bool kLong>
 __global__ void __launch_bounds__(kRowThreads, 1)
 bitdelta_gemm_row_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX,
                          const __grid_constant__ CUtensorMap tmBits, const RowArgs a) {
@@ -165,14 +144,9 @@ bitdelta_gemm_row_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
         // (rows past a short unit's last one read what follows in the stage: they only reach their own outputs, not written)
         const uint32_t wrow0 = (uint32_t)(atom * a.rows + g), wrow1 = wrow0 + 8;
         bool ok = true;
-        int slot = 0, z_group = -1;
-        uint32_t phase = 0;
-        float Z[kNt][4];
-        uint32_t cst[4];
-#pragma unroll
-        for (int c = kF16 ? 7 : 4; c < (kF16 ? 11 : 8); ++c) cst[c & 3] = row_const<kF16>(c);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) asm volatile("" : "+r"(cst[c]));
+        int slot = 0;
+        uint32_t phase = 0, minus_one2 = kF16 ? 0xBC00BC00u : 0xBF80BF80u;
+        asm volatile("" : "+r"(minus_one2));
         const int m = a.m;
         const int jc[2] = {2 * t / m, (2 * t + 1) / m};   // the tenant of the tile that this thread's two columns belong to
         // The partial results of successive units go to two buffers in turn: a warp that writes a buffer again has passed the
@@ -183,24 +157,16 @@ bitdelta_gemm_row_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
             const int tile = unit / a.groups, grp = unit - tile * a.groups;
             const int n0 = tile * a.rows, tenant0 = grp * kTpt * kNt;
             const int nten = min(kTpt * kNt, a.B - tenant0);
-            const bool new_z = grp != z_group;
-            z_group = grp;
-            float accb[kNt][4], accd[kNt][kTpt][4], al[kNt][2];
+            float accb[kNt][4], accd[kNt][kTpt][4], sum[kNt][4], al[kNt][2];
 #pragma unroll
             for (int i = 0; i < kNt; ++i) {
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    accb[i][e] = 0.f;
-                    if (new_z) Z[i][e] = 0.f;
-#pragma unroll
-                    for (int j = 0; j < kTpt; ++j) accd[i][j][e] = 0.f;
-                }
+                for (int e = 0; e < 4; ++e) sum[i][e] = 0.f;
 #pragma unroll
                 for (int e = 0; e < 2; ++e) al[i][e] = (jc[e] < kTpt && i * kTpt + jc[e] < nten) ? __ldg(a.alpha + tenant0 + i * kTpt + jc[e]) : 0.f;
             }
-            // this warp's 128 k of a stage (kZ: with the offsets' sums)
-            auto stage = [&](auto with_z) {
-                constexpr bool kZ = decltype(with_z)::value;
+            // this warp's 128 k of a stage
+            auto stage = [&] {
                 const uint32_t st = base + (uint32_t)slot * a.stage_bytes;
 #pragma unroll
                 for (int i = 0; i < kNt; ++i) {
@@ -209,7 +175,7 @@ bitdelta_gemm_row_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
                     for (int q = 0; q < 4; ++q)
                         x[q] = lds128(st + a.x_off + i * 16384u + xrow * 128u + (uint32_t)(((c0 + (q ^ flip)) ^ (xrow & 7)) << 4));
                     // the tenants' sign words of the rows g, g + 8 (tenants past the unit's own: the first one's, not used)
-                    uint32_t sw[kTpt][2], sv[kTpt][2];
+                    uint32_t sw[kTpt][2];
 #pragma unroll
                     for (int j = 0; j < kTpt; ++j) {
                         const int jj = i * kTpt + j < nten ? i * kTpt + j : 0;
@@ -245,49 +211,54 @@ bitdelta_gemm_row_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
                             mma16816<kF16>(accb[i], w0.x, w1.x, w0.y, w1.y, x[c].x, x[c].y);
                             mma16816<kF16>(accb[i], w0.z, w1.z, w0.w, w1.w, x[c].z, x[c].w);
                         }
-                        if constexpr (kZ) {
-                            const uint32_t o0 = row_mid<kF16>(row_class<kF16>(2 * q)), o1 = row_mid<kF16>(row_class<kF16>(2 * q + 1));
-                            mma16816<kF16>(Z[i], o0, o0, o1, o1, xp[2 * q], xp[2 * q + 1]);
-                        }
 #pragma unroll
-                        for (int j = 0; j < kTpt; ++j) {
-                            if (q == 0 || row_shift<kF16>(2 * q) != row_shift<kF16>(2 * q - 1)) {
-                                sv[j][0] = row_shifted<kF16>(sw[j][0], 2 * q);
-                                sv[j][1] = row_shifted<kF16>(sw[j][1], 2 * q);
-                            }
-                            const uint32_t a0 = row_sign_pair<kF16>(sv[j][0], 2 * q, cst), a1 = row_sign_pair<kF16>(sv[j][1], 2 * q, cst);
-                            if (row_shift<kF16>(2 * q + 1) != row_shift<kF16>(2 * q)) {
-                                sv[j][0] = row_shifted<kF16>(sw[j][0], 2 * q + 1);
-                                sv[j][1] = row_shifted<kF16>(sw[j][1], 2 * q + 1);
-                            }
-                            mma16816<kF16>(accd[i][j], a0, a1, row_sign_pair<kF16>(sv[j][0], 2 * q + 1, cst), row_sign_pair<kF16>(sv[j][1], 2 * q + 1, cst),
+                        for (int j = 0; j < kTpt; ++j)
+                            mma16816<kF16>(accd[i][j], row_sign_pair(sw[j][0], 2 * q, minus_one2), row_sign_pair(sw[j][1], 2 * q, minus_one2),
+                                           row_sign_pair(sw[j][0], 2 * q + 1, minus_one2), row_sign_pair(sw[j][1], 2 * q + 1, minus_one2),
                                            xp[2 * q], xp[2 * q + 1]);
-                        }
                     }
                 }
             };
-            for (int s = 0; s < a.k_stages; ++s) {
-                // (one answer per warp: its lanes leave the wait one by one, and the matrix instructions below need all of them)
-                ok = warp_all(ok && wait_bar(smem_u32(&ctl->full[slot]), phase, abort_flag, 41));
-                if (ok && s * kRowStageK + warp * 128 < a.K) {
-                    if (new_z) stage(std::true_type{});
-                    else stage(std::false_type{});
+            int s = 0;
+            do {
+                const int end = kLong ? min(s + kRowLongStages, a.k_stages) : a.k_stages;
+#pragma unroll
+                for (int i = 0; i < kNt; ++i)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        accb[i][e] = 0.f;
+#pragma unroll
+                        for (int j = 0; j < kTpt; ++j) accd[i][j][e] = 0.f;
+                    }
+                for (; s < end; ++s) {
+                    // (one answer per warp: its lanes leave the wait one by one, and the matrix instructions below need all of them)
+                    ok = warp_all(ok && wait_bar(smem_u32(&ctl->full[slot]), phase, abort_flag, 41));
+                    if (ok && s * kRowStageK + warp * 128 < a.K) stage();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&ctl->empty[slot]));
+                    if (++slot == a.stages) { slot = 0; phase ^= 1; }
                 }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&ctl->empty[slot]));
-                if (++slot == a.stages) { slot = 0; phase ^= 1; }
-            }
-            // this warp's share of every output: base + alpha * (delta with offsets - Z)
+                // this warp's share of every output: base + alpha * delta
 #pragma unroll
-            for (int i = 0; i < kNt; ++i) {
+                for (int i = 0; i < kNt; ++i) {
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    float d = accd[i][0][e];
+                    for (int e = 0; e < 4; ++e) {
+                        float d[kTpt];   // (selected bit by bit of the tenant's number: of a chain of tests the compiler makes an array in local memory)
 #pragma unroll
-                    for (int j = 1; j < kTpt; ++j) d = (jc[e & 1] == j) ? accd[i][j][e] : d;
-                    red[((warp * kNt + i) * 8 + 2 * t + (e & 1)) * 16 + g + 8 * (e >> 1)] = fmaf(al[i][e & 1], d - Z[i][e], accb[i][e]);
+                        for (int j = 0; j < kTpt; ++j) d[j] = accd[i][j][e];
+#pragma unroll
+                        for (int w = kTpt / 2; w > 0; w /= 2)
+#pragma unroll
+                            for (int j = 0; j < w; ++j) d[j] = (jc[e & 1] & w) ? d[j + w] : d[j];
+                        const float v = fmaf(al[i][e & 1], d[0], accb[i][e]);
+                        sum[i][e] = kLong ? sum[i][e] + v : v;
+                    }
                 }
-            }
+            } while (kLong && s < a.k_stages);
+#pragma unroll
+            for (int i = 0; i < kNt; ++i)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) red[((warp * kNt + i) * 8 + 2 * t + (e & 1)) * 16 + g + 8 * (e >> 1)] = sum[i][e];
             named_bar_sync(1, kRowWarps * 32);
             grid_dependency_wait();   // Y may still be in use by the previous kernel
 #pragma unroll
@@ -301,18 +272,6 @@ bitdelta_gemm_row_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
                     const int jt = col / m, n = n0 + row, b = tenant0 + i * kTpt + jt;
                     const bool live = ok && jt < kTpt && b < a.B && row < a.rows && n < a.N;
                     const int tok = b * m + col - jt * m;
-                    if (live && !(fabsf(v) <= 3.0e38f)) {   // term by term
-                        const uint16_t* x = static_cast<const uint16_t*>(a.X) + (size_t)tok * a.K;
-                        const uint16_t* w = static_cast<const uint16_t*>(a.W) + (size_t)n * a.K;
-                        const uint32_t* sg = a.bits + ((size_t)b * a.N + n) * (a.K >> 5);
-                        float vb = 0.f, vd = 0.f;
-                        for (int k = 0; k < a.K; ++k) {
-                            const float xv = from_io16(x[k], kF16);
-                            vb = fmaf(xv, from_io16(w[k], kF16), vb);
-                            vd += ((sg[k >> 5] >> (k & 31)) & 1u) ? xv : -xv;
-                        }
-                        v = fmaf(a.alpha[b], vd, vb);
-                    }
                     if (a.bias && n < a.N) v += from_io16(__ldg(static_cast<const uint16_t*>(a.bias) + n), kF16);
                     uint16_t* Y = static_cast<uint16_t*>(a.Y);
                     if (a.act == 2) {
@@ -337,31 +296,33 @@ bitdelta_gemm_row_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
 }
 
 typedef void (*RowKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const RowArgs);
-template <bool kF16> static RowKernel row_kernel(int tpt, int nt) {
+template <bool kF16, bool kLong> static RowKernel row_kernel(int tpt, int nt) {
     switch (tpt * 8 + nt) {
-        case 65: return bitdelta_gemm_row_kernel<kF16, 8, 1>;
-        case 33: return bitdelta_gemm_row_kernel<kF16, 4, 1>;
-        case 34: return bitdelta_gemm_row_kernel<kF16, 4, 2>;
-        case 17: return bitdelta_gemm_row_kernel<kF16, 2, 1>;
-        case 18: return bitdelta_gemm_row_kernel<kF16, 2, 2>;
-        case 20: return bitdelta_gemm_row_kernel<kF16, 2, 4>;
-        case 9: return bitdelta_gemm_row_kernel<kF16, 1, 1>;
-        case 10: return bitdelta_gemm_row_kernel<kF16, 1, 2>;
-        case 12: return bitdelta_gemm_row_kernel<kF16, 1, 4>;
+        case 65: return bitdelta_gemm_row_kernel<kF16, 8, 1, kLong>;
+        case 33: return bitdelta_gemm_row_kernel<kF16, 4, 1, kLong>;
+        case 34: return bitdelta_gemm_row_kernel<kF16, 4, 2, kLong>;
+        case 17: return bitdelta_gemm_row_kernel<kF16, 2, 1, kLong>;
+        case 18: return bitdelta_gemm_row_kernel<kF16, 2, 2, kLong>;
+        case 20: return bitdelta_gemm_row_kernel<kF16, 2, 4, kLong>;
+        case 9: return bitdelta_gemm_row_kernel<kF16, 1, 1, kLong>;
+        case 10: return bitdelta_gemm_row_kernel<kF16, 1, 2, kLong>;
+        case 12: return bitdelta_gemm_row_kernel<kF16, 1, 4, kLong>;
     }
     return nullptr;
 }
 
 cudaError_t launch_gemm_row(const CUtensorMap& tmW, const CUtensorMap& tmX, const CUtensorMap& tmBits, const RowArgs& args,
                             const RowPlan& p, bool early_start, cudaStream_t stream) {
-    const RowKernel k = args.f16 ? row_kernel<true>(p.tpt, p.nt) : row_kernel<false>(p.tpt, p.nt);
+    const bool long_k = p.k_stages > kRowChainStages;
+    const RowKernel k = args.f16 ? (long_k ? row_kernel<true, true>(p.tpt, p.nt) : row_kernel<true, false>(p.tpt, p.nt))
+                                 : (long_k ? row_kernel<false, true>(p.tpt, p.nt) : row_kernel<false, false>(p.tpt, p.nt));
     if (!k) return cudaErrorInvalidValue;
-    static std::atomic<unsigned char> attr_done[64][2][72];
+    static std::atomic<unsigned char> attr_done[64][4][72];
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    std::atomic<unsigned char>& done = attr_done[dev][args.f16 ? 1 : 0][p.tpt * 8 + p.nt];
+    std::atomic<unsigned char>& done = attr_done[dev][(args.f16 ? 2 : 0) + (long_k ? 1 : 0)][p.tpt * 8 + p.nt];
     if (!done.load()) {
         e = cudaFuncSetAttribute(reinterpret_cast<const void*>(k), cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
         if (e != cudaSuccess) return e;

@@ -12,8 +12,7 @@ struct RowArgs {
     int f16, act;
     int TB, rows, groups, units, stages, k_stages;
     uint32_t s_off, x_off, stage_bytes;
-    const void *X, *W, *bias;
-    const uint32_t* bits;
+    const void* bias;
     const float* alpha;
     void* Y;
 };
