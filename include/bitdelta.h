@@ -102,8 +102,10 @@ int bitdelta_workspace_init(void* workspace, size_t workspace_bytes, void* cuda_
  *          the device must not share a workspace.
  * m <= 16 selects a decode schedule, larger m the tiled (prefill)
  * schedule (several tenants per tile up to m = 64; pairs of thread blocks with
- * 256-row MMAs for m > 64); all run on tcgen05 tensor cores with TMEM
- * accumulators, and bitdelta_gemm_plan tells which one a shape gets.  Shapes
+ * 256-row MMAs for m > 64), which run on tcgen05 tensor cores with TMEM
+ * accumulators; few tenants or small products with m <= 8 run on the row-stream
+ * kernel instead (mma.sync).  bitdelta_gemm_row_stream tells which shapes those
+ * are, bitdelta_gemm_plan which schedule the others get.  Shapes
  * whose K is not a multiple of 128 take the tiled schedule for every m, or a plain
  * CUDA-core kernel: with K < 128, one token against a small matrix, or without
  * the workspace that the tiled schedule needs.
@@ -113,7 +115,7 @@ int bitdelta_workspace_init(void* workspace, size_t workspace_bytes, void* cuda_
  * Row-stream shapes (bitdelta_gemm_row_stream; m <= 8) keep X as it is in both terms and
  * take any magnitude.
  * Precision of X in the decode schedules (other m <= 16): there the delta term runs on
- * a narrow-float tensor path.  bitdelta_gemm_plan tells which of two a shape gets.
+ * a narrow-float tensor path.  bitdelta_gemm_plan tells which of two such a shape gets.
  * 4-bit schedules (plan codes 7, 8; m <= 8, calls without options): every group
  * of 32 consecutive k of a token row is held as 16-bit fixed point relative to the
  * group's largest magnitude.  Values within a factor 2^8 of it are exact; smaller
@@ -233,10 +235,12 @@ int bitdelta_gemm_host(const void* X_host, const void* W_base_host, const uint32
  * is one 128-row tile of W_base for one group of TB tenants (decode schedules) or one tenant's token tile
  * (tiled schedule), a k-step is 128 k; item = unit * P + k-step.
  *
- * bitdelta_gemm_row_stream returns 1 for the shapes (few tenants, or small; m <= 8; calls with options: a somewhat
- * wider range) that run on the row-stream kernel instead: one launch, no scratch, a block per few weight rows with all
- * of K.  bitdelta_gemm_plan reports the schedule that it stands
- * in for, which the same call takes with BITDELTA_ROW=0 in the environment.
+ * bitdelta_gemm_row_stream returns 1 for the shapes (few tenants, or small; m <= 8) that a plain call (bitdelta_gemm)
+ * runs on the row-stream kernel instead: one launch, no scratch, a block per few weight rows with all of K.
+ * bitdelta_gemm_plan reports the schedule that it stands in for, which the same call takes with BITDELTA_ROW=0 in the
+ * environment.  bitdelta_gemm_row_stream_ex answers for a call of bitdelta_gemm_ex with these options (dtype and act codes as
+ * there, has_bias nonzero: with a bias), whose range differs: row-stream calls take activations of any magnitude, the other
+ * calls of m <= 16 have the range that bitdelta_gemm states.
  *
  * bitdelta_gemm_plan fills info[0 .. BITDELTA_PLAN_INFO_INTS-1] (host pointer):
  *   [0] schedule: 0 tiled, 1 decode with a pre-pass activation split, 2 decode with the in-kernel split,
@@ -263,6 +267,7 @@ int bitdelta_gemm_host(const void* X_host, const void* W_base_host, const uint32
 #define BITDELTA_PLAN_INFO_INTS 16
 int bitdelta_gemm_plan(int B, int m, int N, int K, int num_sms, int* info);
 int bitdelta_gemm_row_stream(int B, int m, int N, int K, int num_sms);
+int bitdelta_gemm_row_stream_ex(int B, int m, int N, int K, int dtype, int has_bias, int act, int num_sms);
 int bitdelta_gemm_plan_cta_items(int B, int m, int N, int K, int num_sms, int cta, int* first, int* end);
 int bitdelta_gemm_plan_item_cta(int B, int m, int N, int K, int num_sms, int item);
 

@@ -26,7 +26,7 @@ EXPORTS = (
     "bitdelta_pack", "bitdelta_unpack", "bitdelta_compress_workspace_bytes", "bitdelta_compress",
     "bitdelta_gemm_workspace_bytes", "bitdelta_workspace_init",
     "bitdelta_gemm", "bitdelta_gemm_ex", "bitdelta_gemm_noalloc", "bitdelta_gemm_simt", "bitdelta_gemm_host_arena_bytes", "bitdelta_gemm_host",
-    "bitdelta_gemm_plan", "bitdelta_gemm_row_stream", "bitdelta_gemm_plan_cta_items", "bitdelta_gemm_plan_item_cta",
+    "bitdelta_gemm_plan", "bitdelta_gemm_row_stream", "bitdelta_gemm_row_stream_ex", "bitdelta_gemm_plan_cta_items", "bitdelta_gemm_plan_item_cta",
     "bitdelta_last_device_status", "bitdelta_kernel_launch_count", "bitdelta_status_string", "bitdelta_selftest_timeout",
 )
 
@@ -86,6 +86,7 @@ def load_library():
     lib.bitdelta_gemm_host.argtypes = [vp, vp, vp, vp, vp, ci, ci, ci, ci, vp, sz, vp]
     lib.bitdelta_gemm_plan.argtypes = [ci, ci, ci, ci, ci, ctypes.POINTER(ci)]
     lib.bitdelta_gemm_row_stream.argtypes = [ci, ci, ci, ci, ci]
+    lib.bitdelta_gemm_row_stream_ex.argtypes = [ci, ci, ci, ci, ci, ci, ci, ci]
     lib.bitdelta_gemm_plan_cta_items.argtypes = [ci, ci, ci, ci, ci, ci, ctypes.POINTER(ci), ctypes.POINTER(ci)]
     lib.bitdelta_gemm_plan_item_cta.argtypes = [ci, ci, ci, ci, ci, ci]
     lib.bitdelta_last_device_status.argtypes = [vp, ctypes.POINTER(ci)]
@@ -253,9 +254,11 @@ def gemm_plan(B: int, m: int, N: int, K: int, num_sms: int = 148) -> dict:
     return dict(zip(PLAN_FIELDS, list(info)))
 
 
-def gemm_row_stream(B: int, m: int, N: int, K: int, num_sms: int = 148) -> bool:
-    """Whether bitdelta_gemm runs this shape on the row-stream kernel (gemm_plan then reports what that stands in for)."""
-    return bool(load_library().bitdelta_gemm_row_stream(B, m, N, K, num_sms))
+def gemm_row_stream(B: int, m: int, N: int, K: int, num_sms: int = 148, fp16: bool = False, bias: bool = False,
+                    act: str = "none", wide_range: bool = False) -> bool:
+    """Whether a call of this shape with these options runs on the row-stream kernel (gemm_plan then reports what that stands in for)."""
+    return bool(load_library().bitdelta_gemm_row_stream_ex(B, m, N, K, int(fp16) | (DTYPE_WIDE_RANGE if wide_range else 0),
+                                                           int(bias), ACTS[act], num_sms))
 
 
 def gemm_plan_cta_items(B: int, m: int, N: int, K: int, cta: int, num_sms: int = 148):

@@ -195,6 +195,9 @@ bool take_row_kernel(int B, int m, int N, int K, int sms, bool plain, int cluste
            !getenv("BITDELTA_FP4_COOP");
 }
 
+// Whether a call has no options (the 4-bit decode kernel takes none).
+bool is_plain(int dtype, bool has_bias, int act) { return dtype == BITDELTA_DTYPE_BF16 && !has_bias && act == BITDELTA_ACT_NONE; }
+
 // Encoded tensor maps, kept per (kind, pointer, shape, box): encoding one costs a microsecond or two of host time,
 // a GEMM call needs three or four, and a serving loop calls with the same few weight and activation buffers.
 struct MapKey {
@@ -366,7 +369,7 @@ int bitdelta_gemm_ex(const void* X, const void* W_base, const uint32_t* bits, co
     if (st != BITDELTA_OK) return st;
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
 
-    const bool plain = !f16 && act == BITDELTA_ACT_NONE && bias == nullptr;   // (the 4-bit decode kernel takes no options)
+    const bool plain = is_plain(dtype, bias != nullptr, act);
     bd::Plan p = bd::make_plan(B, m, N, K, d.sms, tb_override(), whole_override(), true, wide, plain);
     if (!wide && p.ok && workspace && workspace_bytes >= p.ws_bytes && aligned16(workspace) && take_row_kernel(B, m, N, K, d.sms, plain, p.cluster)) {
         // (the row-stream kernel needs no scratch; a call that is refused for its workspace stays refused)
@@ -560,9 +563,15 @@ int bitdelta_gemm_plan(int B, int m, int N, int K, int num_sms, int* info) {
 }
 
 int bitdelta_gemm_row_stream(int B, int m, int N, int K, int num_sms) {
+    return bitdelta_gemm_row_stream_ex(B, m, N, K, BITDELTA_DTYPE_BF16, 0, BITDELTA_ACT_NONE, num_sms);
+}
+
+int bitdelta_gemm_row_stream_ex(int B, int m, int N, int K, int dtype, int has_bias, int act, int num_sms) {
     if (B <= 0 || m <= 0 || N <= 0 || K <= 0 || (K % 32) != 0 || num_sms <= 0) return 0;
-    const bd::Plan p = bd::make_plan(B, m, N, K, num_sms, tb_override(), whole_override());
-    return p.ok && take_row_kernel(B, m, N, K, num_sms, true, p.cluster) ? 1 : 0;
+    if ((dtype & BITDELTA_DTYPE_WIDE_RANGE) != 0) return 0;
+    const bool plain = is_plain(dtype, has_bias != 0, act);
+    const bd::Plan p = bd::make_plan(B, m, N, K, num_sms, tb_override(), whole_override(), true, false, plain);
+    return p.ok && take_row_kernel(B, m, N, K, num_sms, plain, p.cluster) ? 1 : 0;
 }
 
 int bitdelta_gemm_plan_cta_items(int B, int m, int N, int K, int num_sms, int cta, int* first, int* end) {
