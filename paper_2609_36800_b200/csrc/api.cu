@@ -190,7 +190,7 @@ bool take_row_kernel(int B, int m, int N, int K, int sms, bool plain, int cluste
     if (e && e[0] == '0') return false;
     const bd::RowPlan p = bd::make_row_plan(B, m, N, K, sms);
     if (e && e[0] == '1') return p.ok;
-    if (!bd::row_kernel_pays(p, B, N, K, plain, cluster)) return false;
+    if (!bd::row_kernel_pays(p, B, m, N, K, plain, cluster)) return false;
     return bd::fp4_mode() == 2 && bd::cluster_enabled() && !getenv("BITDELTA_FP4_INKERNEL") && !getenv("BITDELTA_FP4_RESIDENT") &&
            !getenv("BITDELTA_FP4_COOP");
 }

@@ -69,9 +69,20 @@ inline RowPlan make_row_plan(int B, int m, int N, int K, int num_sms) {
 // Calls with options or binary16 operands have the slower 8-bit kernel as the alternative: up to 68 M (4 x 1 x 4096 x 4096
 // binary16 12.3 / 14.8, 4 x 8 17.5 / 20.5; beyond, 8 x 1 x 1024 x 8448 with a gate 14.2 / 13.3).  Where the 4-bit kernel's clusters of two or four blocks apply (`cluster`), it is ahead
 // from 32 M on (3 x 1 x 2048 x 4096 8.5 / 7.9, 4 x 1 x 2816 x 4096 10.2 / 9.5; without clusters 8 x 1 x 2048 x 2816 10.2 / 14.4).
-inline bool row_kernel_pays(const RowPlan& p, int B, int N, int K, bool plain, int cluster) {
+// Within that, three kinds of call are left to the others (`cols`: token columns x rows computed, in whole rounds, x K in whole stages):
+//   * units of four activation tiles in more than seven rounds: a unit's two barriers and its partial sums cost ~1 us (19 x 5 x 512 x
+//     3642 15.9 / 11.2, 9 x 6 x 512 x 7192 18.9 / 16.0; in seven rounds 11 x 8 x 1024 x 4804 16.8 / 17.8);
+//   * a second round that is mostly empty, with much to compute (binary16 and gate, 12 x 1 x 3200 x 1220 14.1 / 13.0);
+//   * two tenants of five tokens and more (options: eight), large, with the last round partly empty: ~1 us of MMA time per stage,
+//     whatever the rows (2 x 8 x 11008 x 5632 31.2 / 28.9, 2 x 6 x 8192 x 8192 31.3 / 29.3; full rounds: 2 x 8 x 14336 x 11008 62.0 / 67.5).
+inline bool row_kernel_pays(const RowPlan& p, int B, int m, int N, int K, bool plain, int cluster) {
+    if (!p.ok) return false;
+    const long long rounds = (p.units + p.grid - 1) / p.grid, rows = rounds * 16 * p.grid;
+    const long long cols = (long long)p.tpt * p.nt * rows * p.k_stages * kRowStageK;
+    if (B <= 2) return !(B == 2 && m >= (plain ? 5 : 8) && rounds >= 3 && 10ll * N < 9 * rows && cols > 110000000ll);
+    if ((p.nt == 4 && rounds > 7) || (rounds >= 2 && cols > 140000000ll)) return false;
     const long long limit = !plain ? 68000000ll : (cluster == 2 || cluster == 4) ? 32000000ll : 48000000ll;
-    return p.ok && (B <= 2 || (long long)p.tpt * p.nt * p.groups * N * K <= limit);
+    return (long long)p.tpt * p.nt * p.groups * N * K <= limit;
 }
 
 }  // namespace bd

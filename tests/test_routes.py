@@ -32,3 +32,14 @@ def test_calls_clamp_and_flag_large_activations_as_the_query_says(options, row, 
     bd.gemm(X, W, bits, torch.ones(B, device="cuda"), bias=bias, act=options.get("act", "none"))
     assert bd.gemm_row_stream(B, m, N, K, **options) == (row == "1")
     assert bd.last_device_status()[0] == (0 if row == "1" else bd.binding.STATUS_RANGE)
+
+
+@pytest.mark.parametrize("shape,plain,options", [   # B, m, N, K
+    ((19, 5, 3642, 512), False, False), ((9, 6, 7192, 512), False, False), ((10, 5, 3274, 1024), True, True),   # eight, ten, five rounds
+    ((12, 1, 1220, 3200), False, False), ((9, 1, 1550, 2432), False, True),                                      # a second round of six units
+    ((2, 8, 5632, 11008), False, False), ((2, 6, 8192, 8192), False, True), ((2, 8, 11008, 14336), True, True),  # rounds partly empty, full
+    ((2, 4, 8192, 8192), True, True), ((1, 8, 8192, 8192), True, True),
+], ids=str)
+def test_row_stream_range(shape, plain, options):
+    assert bd.gemm_row_stream(*shape) == plain
+    assert bd.gemm_row_stream(*shape, fp16=True, bias=True, act="silu_gate") == options
