@@ -206,21 +206,33 @@ inline Plan make_plan(int B, int m, int N, int K, int num_sms, int tb_override =
         p.slot_floats = (size_t)kTileN * p.TB * m;
     } else {
         p.TB = 1;
-        // CTA pairs take up to 192 tokens a tile (two operand buffers are left beside 384 accumulator columns), single blocks
-        // 128; a tenant's tokens are spread evenly over its tiles.  The tiles' loads from L2 weigh on the schedule (31 bytes per
-        // cycle and multiprocessor at 128 tokens), and a half-empty last tile costs as much as a full one: 4 x 512 x 4096 x
-        // 4096 in tiles of 128: 103.5 us, of 176: 97.7; 4 x 130: 53.4 (two of 128) and 34.5 (one of 144); 2 x 300 x 4096 x
-        // 11008 binary16 with a gate: 115.9 (three of 128) and 95.9 (two of 160).
-        const bool pairs = allow_pair && pair_enabled() && m > 64 && (p.n_tiles % 2) == 0 && num_sms >= 2;
-        p.m_tiles = (m + (pairs ? kMaxTokTile : 128) - 1) / (pairs ? kMaxTokTile : 128);
+        // Single blocks take up to 128 tokens a tile, in steps of 16; CTA pairs up to 192 (two operand buffers are left beside 384
+        // accumulator columns), in steps of 32: the shapes of 256-row MMAs (cta_group::2).  A tenant's tokens are spread evenly
+        // over its tiles.
+        p.m_tiles = (m + 127) / 128;
         p.tok_tile = round_up((m + p.m_tiles - 1) / p.m_tiles, 16);
         p.m_tiles = (m + p.tok_tile - 1) / p.tok_tile;
+        if (allow_pair && pair_enabled() && m > 64 && (p.n_tiles % 2) == 0 && num_sms >= 2) {
+            // Pairs with the fewest columns computed, then the fewest tiles (4 x 512 x 4096 x 4096 in four of 128: 119.3 us, in three
+            // of 192: 120.8; 4 x 130 in one of 160: 40.8, two of 128: 61.6), unless single blocks compute an eighth less:
+            // their columns cost 10 to 17 % more (70 tokens as 96 or 80: 33.0 and 32.2; 193 as 256 or 224: 63.6 and 61.3; but 400
+            // as 480 or 448: 102.8 and 112.6).
+            int tiles = 0, tile = 0;
+            for (int t = (m + kMaxTokTile - 1) / kMaxTokTile; t <= (m + 127) / 128; ++t) {
+                const int c = round_up((m + t - 1) / t, 32);
+                if (tiles == 0 || (long long)t * c < (long long)tiles * tile) { tiles = t; tile = c; }
+            }
+            if (8ll * tiles * tile < 9ll * p.m_tiles * p.tok_tile) {
+                p.pair = 1;
+                p.tok_tile = tile;
+                p.m_tiles = (m + tile - 1) / tile;
+            }
+        }
         p.groups = B * p.m_tiles;
         p.Nb = p.tok_tile;
         p.Nd = p.tok_tile;
         p.win_rows = 0;
         p.chunk_rows = 16;
-        p.pair = (pairs && p.tok_tile >= 80) ? 1 : 0;
         p.x_rows = p.pair ? p.tok_tile / 2 : p.tok_tile;   // a pair's CTAs stage half of the token tile each
         p.N3 = 0;
         p.convert = 0;

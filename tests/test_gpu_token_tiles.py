@@ -12,13 +12,14 @@ pytestmark = pytest.mark.gpu
 
 # B, m, N, K                 token tile
 SHAPES = [
-    ((1, 129, 256, 384), 144),
+    ((2, 81, 256, 384), 96),
+    ((1, 129, 256, 384), 160),
     ((2, 160, 250, 256), 160),
-    ((1, 176, 256, 640), 176),
+    ((1, 176, 256, 640), 192),
     ((3, 192, 512, 1152), 192),
-    ((1, 193, 256, 128), 112),      # two tiles
-    ((2, 350, 512, 384), 176),
-    ((80, 144, 250, 128), 144),     # more tiles than pairs of blocks: whole tiles, one behind the other
+    ((1, 225, 256, 128), 128),      # two tiles
+    ((2, 350, 512, 384), 192),
+    ((80, 144, 250, 128), 160),     # more tiles than pairs of blocks: whole tiles, one behind the other
     ((1, 577, 256, 416), 160),      # K not a multiple of 128, four tiles
 ]
 

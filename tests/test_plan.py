@@ -133,3 +133,16 @@ def test_work_lists_beyond_the_32_bit_split_arithmetic_are_refused():
     assert bd.load_library().bitdelta_gemm_plan(B, m, N, K, 148, info) == 2
     # just below the limit the plan exists
     assert bd.gemm_plan(B, m, N // 2, K)["units"] * bd.gemm_plan(B, m, N // 2, K)["k_steps"] == 1 << 29
+
+
+@pytest.mark.parametrize("K", [1024, 1056])
+def test_pairs_take_token_tiles_in_steps_of_32(K):
+    # 256-row MMAs over two blocks are documented for N in steps of 32 (128-row ones on one block: of 16)
+    paired = 0
+    for m in (*range(65, 400), 512, 577, 1000, 2048):
+        p = bd.gemm_plan(2, m, 512, K)
+        tiles, tile = p["groups"] // 2, p["token_tile"]
+        assert (tiles - 1) * tile < m <= tiles * tile
+        assert (p["schedule"] == 4 and tile % 32 == 0 and tile <= 192) or (p["schedule"] == 0 and tile % 16 == 0 and tile <= 128), (m, p)
+        paired += p["schedule"] == 4
+    assert paired > 250
