@@ -8,10 +8,20 @@ if ROOT not in sys.path:
     sys.path.insert(0, ROOT)
 
 
+# The decode sizes of these modules run on the row-stream kernel by default, which stands in there for the kernels that they were
+# written for: every test runs on both routes.
+BOTH_ROUTES = ("test_gpu_gemm_ex", "test_zz_no_alloc")
+
+
+def pytest_generate_tests(metafunc):
+    if metafunc.module.__name__ in BOTH_ROUTES:
+        metafunc.parametrize("decode_route", ["default", "others"], indirect=True)
+
+
 @pytest.fixture(autouse=True)
-def tcgen05_decode_kernels(request, monkeypatch):
-    """The tests of the 4-bit decode kernel's default route take it also at the sizes that the row-stream kernel has."""
-    if request.module.__name__ == "test_gpu_fp4":
+def decode_route(request, monkeypatch):
+    """"others": the row-stream kernel is never taken.  (The tests of the 4-bit decode kernel's default route need that, too.)"""
+    if getattr(request, "param", None) == "others" or request.module.__name__ == "test_gpu_fp4":
         monkeypatch.setenv("BITDELTA_ROW", "0")
 
 
