@@ -99,7 +99,8 @@ int bitdelta_workspace_init(void* workspace, size_t workspace_bytes, void* cuda_
  *                            conversion at the end
  * workspace / workspace_bytes : at least bitdelta_gemm_workspace_bytes(B,m,N,K),
  *          prepared once by bitdelta_workspace_init; calls that may overlap on
- *          the device must not share a workspace.
+ *          the device must not share a workspace.  A workspace serves one
+ *          (B,m,N,K), with whatever options; for another it is initialised again.
  * m <= 16 selects a decode schedule, larger m the tiled (prefill)
  * schedule (several tenants per tile up to m = 64; pairs of thread blocks with
  * 256-row MMAs for m > 64), which run on tcgen05 tensor cores with TMEM
@@ -193,7 +194,8 @@ int bitdelta_gemm_ex(const void* X, const void* W_base, const uint32_t* bits, co
  *
  * Arguments and result are those of bitdelta_gemm, without the workspace pair.
  *   - Shapes whose workspace (bitdelta_gemm_workspace_bytes) exceeds the array are refused with
- *     BITDELTA_ERR_WORKSPACE and nothing is launched; use bitdelta_gemm with your own buffer.
+ *     BITDELTA_ERR_WORKSPACE and nothing is launched; use bitdelta_gemm with your own buffer.  (K not a
+ *     multiple of 128: they run on the CUDA-core kernel, which needs no workspace and is far slower.)
  *   - The first call on each device looks up the array's device address (the current device must be
  *     the one the call is for) and may be the moment the CUDA runtime binds this library's device image,
  *     array included, to that device: make that first call at start-up, before the memory plan is

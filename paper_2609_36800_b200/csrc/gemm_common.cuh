@@ -136,8 +136,9 @@ __device__ __forceinline__ Unit unit_info_t(const GemmArgs& a, int unit, int am,
 }
 
 // (v & mask) ^ flip in ONE logic operation, written out: it takes one immediate (the mask), the other constant has to be in a
-// register, and the compiler, seeing two constants, makes two operations of it (8-bit decode, 32 x 8 x 14336 x 4096: 167 us with
-// two, 153 with one; 8 x 1 x 4096 x 22016 with a gate 62.1 and 58.7; 8 x 1 x 4096 x 4096, 4-bit: 14.75 and 14.55).
+// register, and the compiler, seeing two constants, makes two operations of it (two and one, us, in a graph: 8-bit decode, 32 x 8 x
+// 14336 x 4096 169 and 159, 16 x 4 x 4096 x 11008 with bias and gate 64.4 and 61.1; 4-bit flat list, 16 x 4 x 4096 x 11008 53.0 and 51.9.
+// The 4-bit kernel's cluster form takes it for half of its registers only, see there).
 __device__ __forceinline__ uint32_t and_xor(uint32_t v, uint32_t mask, uint32_t flip) {
     uint32_t d;
     asm("lop3.b32 %0, %1, %2, %3, 0x6A;" : "=r"(d) : "r"(v), "r"(mask), "r"(flip));

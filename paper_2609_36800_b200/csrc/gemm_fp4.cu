@@ -1095,7 +1095,7 @@ bitdelta_gemm_fp4_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
                 FT_ADD(3);
             }
         }
-        if (warp == kFWarpEpi0) FT_OUT(16, 8);
+        if (warp == kFWarpEpi0) FT_OUT(16, 8);   // (the sums of cut tiles come after the roles and are in none of them)
         if (!ok) {
             // This warp left on an abandoned wait; a sibling that passed the same wait a moment earlier may be
             // waiting on the epilogue barrier: release it once (it then sees the flag and leaves too).

@@ -6,8 +6,8 @@
 // activations through shared memory in stages of 1024 k (bulk-tensor copies, 128-byte rows); eight consumer warps take 128 k
 // of a stage each and keep fp32 sums in registers; at the end of a unit the eight partial sums are added in shared memory.
 // There is no activation pre-pass, no tensor-memory hand-over, no workspace and no sum across blocks: for few tenants
-// those latencies are most of a call of the other decode kernels (1 x 8 x 1024 x 1024: 2.3 us, 5.6 there; 8 x 1 x 2048 x 2048:
-// 6.7 and 13.6; 1 x 1 x 4096 x 4096: 8.7 and 10.5, 4.1 TB/s).
+// those latencies are most of a call of the other decode kernels (1 x 8 x 1024 x 1024: 2.3 us, 5.3 there; 8 x 1 x 2048 x 2048:
+// 6.2 and 14.3; 1 x 1 x 4096 x 4096: 8.3 and 10.3, 4.3 TB/s).
 //
 // The products run on mma.sync (m16n8k16, the weights on the 16-row side), because its A operand comes from registers, where the
 // decoded signs are; that path is a quarter as fast as tcgen05, which is what limits the kernel to few tenants.
@@ -151,7 +151,7 @@ bitdelta_gemm_row_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
         const int jc[2] = {2 * t / m, (2 * t + 1) / m};   // the tenant of the tile that this thread's two columns belong to
         // The partial results of successive units go to two buffers in turn: a warp that writes a buffer again has passed the
         // barrier of the unit between, which the others reach only after they have read it, so one barrier a unit is enough
-        // (2 x 1 x 4096 x 4096 10.5 -> 9.9 us, 2 x 4 x 1024 x 8192 8.4 -> 7.8).  Four activation tiles leave no room for two.
+        // (2 x 1 x 4096 x 4096 10.5 -> 9.9 us then, 2 x 4 x 1024 x 8192 8.4 -> 7.8).  Four activation tiles leave no room for two.
         for (int unit = (int)blockIdx.x, odd = 0; unit < a.units; unit += (int)gridDim.x, odd ^= 1) {
             float* red = reinterpret_cast<float*>(smem + red_off) + (kRedBufs == 2 ? odd * kRedFloats : 0);
             const int tile = unit / a.groups, grp = unit - tile * a.groups;

@@ -61,14 +61,15 @@ inline RowPlan make_row_plan(int B, int m, int N, int K, int num_sms) {
 }
 
 // Where the row-stream kernel is taken by default: one or two tenants, or up to 48 M signs including the tenant columns computed
-// for nothing.  Its MMAs cost ~1.2 us per tenant at 4096 x 4096, the others' latencies are the same whatever the size.
-// Measured (us, row-stream / the others): 1 x 1 x 4096 x 4096 8.7 / 10.5, 1 x 8 x 4096 x 11008 17.2 / 22.9, 2 x 1 x 4096 x 4096
-// 9.9 / 10.9, 2 x 8 11.3 / 13.5, 8 x 1 x 2048 x 2048 6.7 / 13.6, 8 x 8 x 1024 x 1024 4.2 / 12.4, 4 x 2 x 5632 x 2048 11.1 / 18.3,
-// 16 x 1 x 2048 x 768 6.3 / 14.9; beyond: 4 x 1 x 4096 x 4096 12.9 / 11.9, 8 x 1 17.4 / 14.9, 28 x 1 x 6400 x 816 28.3 / 21.2.
-// (In the other direction a few are left to the others that it would win: 32 x 1 x 2048 x 1024 11.8 / 16.9.)
-// Calls with options or binary16 operands have the slower 8-bit kernel as the alternative: up to 68 M (4 x 1 x 4096 x 4096
-// binary16 12.3 / 14.8, 4 x 8 17.5 / 20.5; beyond, 8 x 1 x 1024 x 8448 with a gate 14.2 / 13.3).  Where the 4-bit kernel's clusters of two or four blocks apply (`cluster`), it is ahead
-// from 32 M on (3 x 1 x 2048 x 4096 8.5 / 7.9, 4 x 1 x 2816 x 4096 10.2 / 9.5; without clusters 8 x 1 x 2048 x 2816 10.2 / 14.4).
+// for nothing.  Its MMAs cost ~1.1 us per tenant at 4096 x 4096, the others' latencies are the same whatever the size.
+// Measured (us, row-stream / the others, in a graph): 1 x 1 x 4096 x 4096 8.4 / 10.5, 1 x 8 x 4096 x 11008 15.7 / 21.6, 2 x 1 x 4096 x 4096
+// 9.6 / 11.0, 2 x 8 10.6 / 13.0, 8 x 1 x 2048 x 2048 6.3 / 13.4, 8 x 8 x 1024 x 1024 3.5 / 12.6, 4 x 2 x 5632 x 2048 9.9 / 18.4,
+// 16 x 1 x 2048 x 768 5.2 / 14.1; beyond: 4 x 1 x 4096 x 4096 12.1 / 11.7, 8 x 1 16.5 / 14.2, 28 x 1 x 6400 x 816 23.2 / 19.9.
+// (In the other direction some are left to the others that it would win: 32 x 1 x 2048 x 1024 9.3 / 16.7.)
+// Calls with options or binary16 operands have the slower 8-bit kernel as the alternative: up to 68 M (binary16, bias, gate: 4 x 1 x
+// 4096 x 4096 12.8 / 14.6, 4 x 8 16.6 / 21.5; beyond, 28 x 1 x 6400 x 816 23.5 / 19.5).  Where the 4-bit kernel's clusters of two or four
+// blocks apply (`cluster`), it is ahead from 32 M on (3 x 1 x 2048 x 4096 8.3 / 7.8, 4 x 1 x 2816 x 4096 10.0 / 9.3; without clusters
+// 8 x 1 x 2048 x 2816 9.8 / 14.9).
 // Within that, three kinds of call are left to the others (`cols`: token columns x rows computed, in whole rounds, x K in whole stages):
 //   * units of four activation tiles in more than seven rounds: a unit's two barriers and its partial sums cost ~1 us (19 x 5 x 512 x
 //     3642 15.9 / 11.2, 9 x 6 x 512 x 7192 18.9 / 16.0; in seven rounds 11 x 8 x 1024 x 4804 16.8 / 17.8);

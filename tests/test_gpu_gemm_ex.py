@@ -30,7 +30,7 @@ def run_ex(X, W, bits, alpha, bias, dtype, act):
 
 
 # every schedule: in-kernel split (m small), pre-pass split, tiled, cut tiles (split-K fix-up), teams,
-# ragged N, CUDA-core fallback (K not a multiple of 128)
+# ragged N, CUDA-core kernel (K < 128)
 SHAPES = [
     (1, 1, 128, 128),
     (8, 1, 1024, 1024),
@@ -40,7 +40,7 @@ SHAPES = [
     (7, 9, 256, 256),
     (2, 17, 256, 384),
     (2, 100, 300, 640),
-    (2, 130, 256, 512),     # token tiles of 128 and two W_base tiles: the schedule on CTA pairs
+    (2, 130, 256, 512),     # one token tile of 160 and two W_base tiles: the schedule on CTA pairs
     (2, 90, 256, 384),      # CTA pairs, token tile of 96
     (5, 20, 384, 512),
     (3, 33, 264, 384),

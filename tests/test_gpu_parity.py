@@ -119,7 +119,7 @@ def test_small_shapes_match_oracle(shape):
 
 
 @pytest.mark.parametrize("shape", [(2, 3, 96, 96), (1, 20, 130, 224), (3, 1, 64, 32)])
-def test_k_not_multiple_of_128_uses_cuda_core_kernel(shape):
+def test_k_not_multiple_of_128(shape):
     B, m, N, K = shape
     wl = synth.Workload("t", B=B, m=m, K=K, N=N, seed=5)
     X, W, bits, alpha = synth.make_inputs(wl)
