@@ -194,8 +194,9 @@ int bitdelta_gemm_ex(const void* X, const void* W_base, const uint32_t* bits, co
  *
  * Arguments and result are those of bitdelta_gemm, without the workspace pair.
  *   - Shapes whose workspace (bitdelta_gemm_workspace_bytes) exceeds the array are refused with
- *     BITDELTA_ERR_WORKSPACE and nothing is launched; use bitdelta_gemm with your own buffer.  (K not a
- *     multiple of 128: they run on the CUDA-core kernel, which needs no workspace and is far slower.)
+ *     BITDELTA_ERR_WORKSPACE and nothing is launched; use bitdelta_gemm with your own buffer.  (Not refused: a
+ *     paired tiled shape that fits on single blocks, which it then takes; and K not a multiple of 128, which
+ *     then runs on the CUDA-core kernel, needs no workspace and is far slower.)
  *   - The first call on each device looks up the array's device address (the current device must be
  *     the one the call is for) and may be the moment the CUDA runtime binds this library's device image,
  *     array included, to that device: make that first call at start-up, before the memory plan is

@@ -352,9 +352,9 @@ int bitdelta_gemm(const void* X, const void* W_base, const uint32_t* bits, const
                             workspace, workspace_bytes, cuda_stream);
 }
 
-int bitdelta_gemm_ex(const void* X, const void* W_base, const uint32_t* bits, const float* alpha, const void* bias,
-                     void* Y, int B, int m, int N, int K, int dtype, int act, void* workspace,
-                     size_t workspace_bytes, void* cuda_stream) {
+// (allow_pair: the tiled schedule may run on pairs of blocks)
+static int run_gemm(const void* X, const void* W_base, const uint32_t* bits, const float* alpha, const void* bias, void* Y, int B, int m, int N,
+                    int K, int dtype, int act, void* workspace, size_t workspace_bytes, void* cuda_stream, bool allow_pair) {
     int st = check_gemm_args(X, W_base, bits, alpha, Y, B, m, N, K);
     if (st != BITDELTA_OK) return st;
     const bool wide = (dtype & BITDELTA_DTYPE_WIDE_RANGE) != 0;
@@ -370,7 +370,7 @@ int bitdelta_gemm_ex(const void* X, const void* W_base, const uint32_t* bits, co
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
 
     const bool plain = is_plain(dtype, bias != nullptr, act);
-    bd::Plan p = bd::make_plan(B, m, N, K, d.sms, tb_override(), whole_override(), true, wide, plain);
+    bd::Plan p = bd::make_plan(B, m, N, K, d.sms, tb_override(), whole_override(), allow_pair, wide, plain);
     if (!wide && p.ok && workspace && workspace_bytes >= p.ws_bytes && aligned16(workspace) && take_row_kernel(B, m, N, K, d.sms, plain, p.cluster)) {
         // (the row-stream kernel needs no scratch; a call that is refused for its workspace stays refused)
         const bd::RowPlan rp = bd::make_row_plan(B, m, N, K, d.sms);
@@ -493,6 +493,12 @@ int bitdelta_gemm_ex(const void* X, const void* W_base, const uint32_t* bits, co
     if (le != cudaSuccess) return BITDELTA_ERR_CUDA;
     g_launches++;
     return BITDELTA_OK;
+}
+
+int bitdelta_gemm_ex(const void* X, const void* W_base, const uint32_t* bits, const float* alpha, const void* bias,
+                     void* Y, int B, int m, int N, int K, int dtype, int act, void* workspace,
+                     size_t workspace_bytes, void* cuda_stream) {
+    return run_gemm(X, W_base, bits, alpha, bias, Y, B, m, N, K, dtype, act, workspace, workspace_bytes, cuda_stream, true);
 }
 
 size_t bitdelta_gemm_host_arena_bytes(int B, int m, int N, int K) {
@@ -640,8 +646,15 @@ int bitdelta_gemm_noalloc(const void* X, const void* W_base, const uint32_t* bit
     if (st != BITDELTA_OK) return st;
     const size_t need = bitdelta_gemm_workspace_bytes(B, m, N, K);
     if (need == 0) return BITDELTA_ERR_SHAPE;
-    if (need > (size_t)BITDELTA_NOALLOC_SCRATCH_BYTES && (K % 128) == 0)   // (other K: the CUDA-core kernel needs no scratch)
-        return BITDELTA_ERR_WORKSPACE;
+    bd::Plan plan = bd::make_plan(B, m, N, K, d.sms, tb_override(), whole_override());
+    bool pairs = true;
+    if (need > (size_t)BITDELTA_NOALLOC_SCRATCH_BYTES && (K % 128) == 0) {   // (other K: the CUDA-core kernel needs no scratch)
+        // (the partial results of pairs' wider token tiles may not fit where those of single blocks do)
+        pairs = false;
+        if (plan.pair) plan = bd::make_plan(B, m, N, K, d.sms, tb_override(), whole_override(), false);
+        else plan.ok = false;
+        if (!plan.ok || plan.ws_bytes > (size_t)BITDELTA_NOALLOC_SCRATCH_BYTES) return BITDELTA_ERR_WORKSPACE;
+    }
 
     // Device address of the scratch array, looked up once per device with that device current.
     static void* scratch_ptr[64] = {};
@@ -659,14 +672,13 @@ int bitdelta_gemm_noalloc(const void* X, const void* W_base, const uint32_t* bit
     }
     // The arrival counters at the start of the scratch have to be zero when the kernel begins; a call
     // that was cut short could have left them otherwise.
-    bd::Plan plan = bd::make_plan(B, m, N, K, d.sms, tb_override(), whole_override());
     if (!plan.ok && (K % 128) == 0) return BITDELTA_ERR_SHAPE;
     if (plan.ok && plan.ws_bytes <= (size_t)BITDELTA_NOALLOC_SCRATCH_BYTES) {
         if (cudaMemsetAsync(scratch, 0, plan.ws_header_bytes, static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess)
             return BITDELTA_ERR_CUDA;
     }
-    return bitdelta_gemm(X, W_base, bits, alpha, Y, B, m, N, K, scratch, (size_t)BITDELTA_NOALLOC_SCRATCH_BYTES,
-                         cuda_stream);
+    return run_gemm(X, W_base, bits, alpha, nullptr, Y, B, m, N, K, BITDELTA_DTYPE_BF16, BITDELTA_ACT_NONE, scratch,
+                    (size_t)BITDELTA_NOALLOC_SCRATCH_BYTES, cuda_stream, pairs);
 }
 
 unsigned long long bitdelta_kernel_launch_count(void) { return g_launches.load(); }

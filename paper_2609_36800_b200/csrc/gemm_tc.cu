@@ -131,6 +131,10 @@ bitdelta_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
     SegIter it{lo, hi, a.P, a.whole_units ? (int)gridDim.x : 0};
     int unit, p0, p1;
 
+    // Pair schedule: columns computed for a unit, a multiple of 32 (cta_group::2); a tenant's last token tile may have fewer than the
+    // others.  Each CTA holds the activations of one half of them, from the first row of its tile on.
+    auto pair_cols = [](const Unit& u) { return (u.ntok + 31) & ~31; };
+
     // Sums the partial results of a cut tile this block was the last to arrive at.  All warps do it when their roles have
     // ended; with one or eight tokens per tenant the epilogue warps do it in place (32 x 8 x 14336 x 4096: 155 us, at the end
     // 170; 16 x 8 x 4096 x 4096: 34.6 and 37.6; but 8 x 12 x 4096 x 4096 29.3 and 26.2, 16 x 4 x 4096 x 11008 with options 66.0
@@ -321,7 +325,7 @@ bitdelta_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
                         if constexpr (kPair) {
                             // this CTA's half of the token tile, counted on the leader's barrier
                             const uint32_t lbar = mapa_shared(bar, 0);
-                            const int xrow = ux.xrow0 + (int)rank * (a.tok_tile / 2);
+                            const int xrow = ux.xrow0 + (int)rank * (pair_cols(ux) / 2);
                             if (ragged && xi.p == a.P - 1) {
                                 tma_load_2d_pair(dst, &tmBits, lbar, 0, xrow);
                                 tma_load_2d_pair(dst + a.x_atom_bytes, &tmBits, lbar, kAtomK, xrow);
@@ -422,9 +426,9 @@ bitdelta_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
         //   decode schedule: one item = all tenants of the unit x 64 k of e5m2 signs (16 columns per
         //                    tenant, 2 MMAs of K=32 per tenant)
         constexpr uint32_t kM = kPair ? 2 * kTileN : kTileN;   // MMA M: both CTAs' weight rows in the pair schedule
-        const uint32_t idesc_base = io_f16 ? make_idesc_f16(kM, (uint32_t)a.Nb) : make_idesc_bf16(kM, (uint32_t)a.Nb);
-        const uint32_t idesc_delta = kDec ? make_idesc_e5m2(kTileN, (uint32_t)a.Nd)
-                                          : (io_f16 ? make_idesc_f16(kM, (uint32_t)a.Nd) : make_idesc_bf16(kM, (uint32_t)a.Nd));
+        uint32_t idesc_base = io_f16 ? make_idesc_f16(kM, (uint32_t)a.Nb) : make_idesc_bf16(kM, (uint32_t)a.Nb);
+        uint32_t idesc_delta = kDec ? make_idesc_e5m2(kTileN, (uint32_t)a.Nd)
+                                    : (io_f16 ? make_idesc_f16(kM, (uint32_t)a.Nd) : make_idesc_bf16(kM, (uint32_t)a.Nd));
         // Descriptor of a tile = descriptor of address 0 plus (address >> 4): addresses stay below
         // 256 KiB, so the sum never carries out of the 14-bit start-address field.
         const uint64_t desc0 = make_smem_desc_sw128(0);
@@ -442,6 +446,7 @@ bitdelta_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
             ok = warp_all(wait_bar(smem_u32(&ctl->accempty), accphase ^ 1, abort_flag, 3));
             if (!ok) break;
             tc_fence_after();
+            if constexpr (kPair) idesc_base = idesc_delta = io_f16 ? make_idesc_f16(kM, (uint32_t)pair_cols(u)) : make_idesc_bf16(kM, (uint32_t)pair_cols(u));
             for (int p = p0; p < p1 && ok; ++p) {
                 {
                     ok = warp_all(wait_bar(smem_u32(&ctl->wfull[stage]), phase, abort_flag, 4));

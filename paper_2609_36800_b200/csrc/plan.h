@@ -213,19 +213,16 @@ inline Plan make_plan(int B, int m, int N, int K, int num_sms, int tb_override =
         p.tok_tile = round_up((m + p.m_tiles - 1) / p.m_tiles, 16);
         p.m_tiles = (m + p.tok_tile - 1) / p.tok_tile;
         if (allow_pair && pair_enabled() && m > 64 && (p.n_tiles % 2) == 0 && num_sms >= 2) {
-            // Pairs with the fewest columns computed, then the fewest tiles (4 x 512 x 4096 x 4096 in four of 128: 119.3 us, in three
-            // of 192: 120.8; 4 x 130 in one of 160: 40.8, two of 128: 61.6), unless single blocks compute an eighth less:
-            // their columns cost 10 to 17 % more (70 tokens as 96 or 80: 33.0 and 32.2; 193 as 256 or 224: 63.6 and 61.3; but 400
-            // as 480 or 448: 102.8 and 112.6).
-            int tiles = 0, tile = 0;
-            for (int t = (m + kMaxTokTile - 1) / kMaxTokTile; t <= (m + 127) / 128; ++t) {
-                const int c = round_up((m + t - 1) / t, 32);
-                if (tiles == 0 || (long long)t * c < (long long)tiles * tile) { tiles = t; tile = c; }
-            }
-            if (8ll * tiles * tile < 9ll * p.m_tiles * p.tok_tile) {
+            // The fewest tiles, spread evenly; the last one computes what is left of the tokens (4 x 512 x 4096 x 4096 as 192 + 192 +
+            // 128: 110.5 us, as four of 128: 117.1; 2 x 1000 113.6 and 115.9; 4 x 130 as 160: 40.5, as two of 128: 62.0).
+            // Single blocks where they compute an eighth less: their columns cost 10 to 17 % more (70 tokens as 96 or 80: 33.0 and
+            // 32.2; but 400 as 480 or 448: 102.8 and 112.6).
+            const int tiles = (m + kMaxTokTile - 1) / kMaxTokTile, tile = round_up((m + tiles - 1) / tiles, 32);
+            const long long cols = (tiles - 1ll) * tile + round_up(m - (tiles - 1) * tile, 32);
+            if (8 * cols < 9ll * p.m_tiles * p.tok_tile) {
                 p.pair = 1;
                 p.tok_tile = tile;
-                p.m_tiles = (m + tile - 1) / tile;
+                p.m_tiles = tiles;
             }
         }
         p.groups = B * p.m_tiles;

@@ -17,7 +17,10 @@ SHAPES = [
     ((2, 160, 250, 256), 160),
     ((1, 176, 256, 640), 192),
     ((3, 192, 512, 1152), 192),
-    ((1, 225, 256, 128), 128),      # two tiles
+    ((1, 193, 256, 128), 128),      # two tiles, the last of 96 columns
+    ((2, 512, 512, 1152), 192),     # 192, 192 and 128, cut across blocks
+    ((1, 385, 256, 416), 160),      # 160, 160 and 96, K not a multiple of 128
+    ((1, 1345, 256, 256), 192),     # seven tiles and one token
     ((2, 350, 512, 384), 192),
     ((80, 144, 250, 128), 160),     # more tiles than pairs of blocks: whole tiles, one behind the other
     ((1, 577, 256, 416), 160),      # K not a multiple of 128, four tiles

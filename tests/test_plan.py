@@ -143,6 +143,9 @@ def test_pairs_take_token_tiles_in_steps_of_32(K):
         p = bd.gemm_plan(2, m, 512, K)
         tiles, tile = p["groups"] // 2, p["token_tile"]
         assert (tiles - 1) * tile < m <= tiles * tile
-        assert (p["schedule"] == 4 and tile % 32 == 0 and tile <= 192) or (p["schedule"] == 0 and tile % 16 == 0 and tile <= 128), (m, p)
-        paired += p["schedule"] == 4
+        if p["schedule"] == 4:
+            assert tile % 32 == 0 and tile <= 192 and tiles == -(-m // 192), (m, p)
+            paired += 1
+        else:
+            assert p["schedule"] == 0 and tile % 16 == 0 and tile <= 128, (m, p)
     assert paired > 250

@@ -74,3 +74,15 @@ def test_shapes_beyond_the_fixed_scratch_are_refused_without_a_launch():
     status = lib.bitdelta_gemm_noalloc(p, p, p, p, p, wl.B, wl.m, wl.N, wl.K, None)
     assert status == 4 and "workspace" in bd.status_string(status)
     assert bd.kernel_launch_count() == before
+
+
+def test_paired_shapes_whose_partial_results_fit_on_single_blocks_only():
+    # three tiles of 160 tokens on pairs: 17 MB of partial results; four of 112 on single blocks: 16
+    B, m, N, K = 1, 432, 2293, 256
+    assert bd.gemm_plan(B, m, N, K)["schedule"] == 4 and bd.gemm_workspace_bytes(B, m, N, K) > bd.binding.NOALLOC_SCRATCH_BYTES
+    X, W, bits, alpha = synth.make_inputs(synth.Workload("e", B=B, m=m, K=K, N=N, seed=36))
+    out = torch.full((B, m, N), float("nan"), dtype=torch.bfloat16, device="cuda")
+    bd.gemm_noalloc(*to_device(X, W, bits, alpha), out)
+    assert bd.last_device_status()[0] == 0
+    max_abs, rel_fro = errors(y_to_f64(out), oracle.gemm(X, W, bits, alpha))
+    assert max_abs <= MAX_ABS_TOL and rel_fro <= REL_FRO_TOL
