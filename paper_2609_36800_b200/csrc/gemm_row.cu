@@ -30,12 +30,12 @@ namespace bd {
 constexpr int kRowWarps = 8;                                  // consumers; warp 8 is the producer
 constexpr int kRowThreads = (kRowWarps + 1) * 32;
 
-// The matrix unit truncates as it accumulates, so a long chain of MMAs drifts.  Up to kRowChainStages stages (eight MMAs per sum and
-// warp each) are one chain; a longer K is added up in chains of kRowLongStages, with rounded additions between them.  Error of the
-// delta's sum against 64 bits, relative, 2 x 8 x 14336 x 1024 in binary16 (the 8-bit kernel's beside it): N(0, 1) 1.7e-7 in one chain
-// (8.2e-7), heavy-tailed (N(0, 1) times exp(1.5 N(0, 1))) 1.5e-6 in one chain, 1.9e-7 in chains of two (1.8e-7).  Time: 1-2 % where
-// the chains are cut, which is why short K are not.
-constexpr int kRowChainStages = 4, kRowLongStages = 2;
+// The matrix unit truncates as it accumulates, so a long chain of MMAs drifts: at most this many stages (of eight MMAs per sum and
+// warp) are one chain, then a rounded addition takes over.  Error of the delta's sum against 64 bits, relative, 2 x 8 x 14336 x 1024 in
+// binary16, in one chain, in chains of four and of two stages (8-bit kernel): N(0, 1) 1.7e-7, 8.6e-8, 8.8e-8 (8.2e-7); heavy-tailed,
+// N(0, 1) times exp(1.5 N(0, 1)), 1.5e-6, 3.1e-7, 1.9e-7 (1.8e-7).  Time, 2 x 1 x 6656 x 9920: 27.4, 27.6, 28.2 us; a form of its own
+// for K within one chain, which does not pay for the additions (2 x 1 x 4096 x 4096 9.3 us, 9.6 with them).
+constexpr int kRowChainStages = 4;
 
 struct RowCtl {
     uint64_t full[kRowMaxStages], empty[kRowMaxStages];
@@ -221,7 +221,7 @@ bitdelta_gemm_row_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
             };
             int s = 0;
             do {
-                const int end = kLong ? min(s + kRowLongStages, a.k_stages) : a.k_stages;
+                const int end = kLong ? min(s + kRowChainStages, a.k_stages) : a.k_stages;
 #pragma unroll
                 for (int i = 0; i < kNt; ++i)
 #pragma unroll
