@@ -103,7 +103,7 @@ int bitdelta_workspace_init(void* workspace, size_t workspace_bytes, void* cuda_
  *          (B,m,N,K), with whatever options; for another it is initialised again.
  * m <= 16 selects a decode schedule, larger m the tiled (prefill)
  * schedule (several tenants per tile up to m = 64; pairs of thread blocks with
- * 256-row MMAs for m > 64), which run on tcgen05 tensor cores with TMEM
+ * 256-row MMAs for most m > 64), which run on tcgen05 tensor cores with TMEM
  * accumulators; few tenants or small products with m <= 8 run on the row-stream
  * kernel instead (mma.sync).  bitdelta_gemm_row_stream tells which shapes those
  * are, bitdelta_gemm_plan which schedule the others get.  Shapes
