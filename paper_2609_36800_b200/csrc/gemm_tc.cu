@@ -703,6 +703,7 @@ bitdelta_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
             for (int p = p0; p < p1 && ok; ++p) {
                 if (p == p0 || !(p & 1)) {
                     ok = wait_bar(smem_u32(&ctl->bfull[bslot]), bphase, abort_flag, 6);
+                    if constexpr (kGrouped) ok = warp_all(ok);   // (one answer per warp: its lanes store to tensor memory together)
                     if (!ok) break;
                 }
                 const uint8_t* bsl = bits_ptr + bslot * a.bslot_bytes + (p & 1) * 16;
@@ -814,7 +815,7 @@ bitdelta_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
                         uint32_t r[32], r2[32];
                         decode_word(w.x, r, minus_one2);
                         decode_word(w.y, r + 16, minus_one2);
-                        ok = wait_bar(aempty_g + (uint32_t)ar.idx * 8, ar.par ^ 1, abort_flag, 7);
+                        ok = warp_all(wait_bar(aempty_g + (uint32_t)ar.idx * 8, ar.par ^ 1, abort_flag, 7));
                         if (!ok) break;
                         tc_fence_after();
                         const uint32_t tbuf = tbuf_g + (uint32_t)ar.idx * (uint32_t)a.aslot_cols;
@@ -967,6 +968,7 @@ bitdelta_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
                 slotp = a.partials + (size_t)slot * a.slot_floats;
             }
             ok = wait_bar(smem_u32(&ctl->accfull), accphase, abort_flag, 8);
+            if constexpr (kGrouped) ok = warp_all(ok);
             if (!ok) break;
             tc_fence_after();
             accphase ^= 1;

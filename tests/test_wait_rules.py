@@ -14,3 +14,12 @@ def test_waits_of_the_row_stream_kernel():
     assert producer.count("wait_bar(") == 1 and "if (lane == 0) {" in producer
     waits = re.findall(r"[^\n]*wait_bar\([^\n]*", consumers)
     assert waits and all("warp_all(" in w for w in waits), waits
+
+
+def test_waits_of_the_several_tenants_roles():
+    # (decode: tcgen05.st behind the sign words' and the operand buffer's wait; epilogue: tcgen05.ld behind the accumulators')
+    src = open(os.path.join(CSRC, "gemm_tc.cu")).read()
+    branch = src[src.index("// warp (grp, quad): the tenants j = grp, grp+2, ..., one buffer of the group's ring each"):]
+    assert re.search(r"wait_bar\(", branch[:branch.index("tmem_st32")]) and "warp_all(wait_bar(aempty_g" in branch[:branch.index("tmem_st32")]
+    for wait in (r"wait_bar\(smem_u32\(&ctl->bfull\[bslot\]\), bphase, abort_flag, 6\);", r"wait_bar\(smem_u32\(&ctl->accfull\), accphase, abort_flag, 8\);"):
+        assert re.search(wait + r"\s+if constexpr \(kGrouped\) ok = warp_all\(ok\);", src), wait
