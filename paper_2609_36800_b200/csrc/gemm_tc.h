@@ -139,6 +139,8 @@ cudaError_t launch_gemm_fp4(const CUtensorMap& tmW, const CUtensorMap& tmBits, c
 int fp4_max_active_clusters(uint32_t smem_bytes, int cluster);
 cudaError_t read_fp4_status(unsigned int out[2]);
 
+cudaError_t read_compress_status(unsigned int out[2]);
+
 // One warp that lets a bounded wait expire after `limit_cycles` (see bitdelta_selftest_timeout).
 cudaError_t launch_selftest_timeout(long long limit_cycles, int site, cudaStream_t stream);
 
