@@ -138,66 +138,59 @@ __global__ void gemm_simt_kernel(const uint16_t* __restrict__ X, const uint16_t*
 // tensor path (K = 32 per instruction, signs decoded four per register), so each bf16 activation
 // is rewritten, once per call, as a chain of four e5m2 pieces: p0 = rn(x), p1 = rn(x - p0), ...
 // Each piece removes three more bits, so x = p0 + p1 + p2 + p3 up to 2^-12 |x| (e5m2 has the
-// exponent range of fp16: magnitudes above 57344 saturate, below 2^-16 vanish).  Elementwise; one
-// thread per group of 32 k.  Inside a group the pieces are stored in the order the sign decode
-// produces: byte slot 4c+i holds k = c + 8i.  Output rows: X8[(b*4 + q)*m + t, :] for piece q.
-__device__ __forceinline__ float e5m2_value(uint8_t v) {
-    return __half2float(__half(__nv_cvt_fp8_to_halfraw(v, __NV_E5M2)));
-}
-__device__ __forceinline__ uint8_t e5m2_round(float v) {
-    return (uint8_t)__nv_cvt_float_to_fp8(v, __NV_SATFINITE, __NV_E5M2);
-}
-
+// exponent range of fp16: magnitudes above 57344 saturate, below 2^-16 vanish).  Elementwise; four
+// neighbouring threads per group of 32 k.  Inside a group the pieces are stored in the order the sign decode
+// produces: byte slot 4c+i holds k = c + 8i; thread u of the four makes the slots of c = 2u and 2u + 1, from
+// pairs of neighbours.  Output rows: X8[(b*4 + q)*m + t, :] for piece q.
+// Bound by latency and, with many rows, by the conversions: eight values a thread, converted in pairs, and no fourth
+// piece where the third leaves nothing (every bfloat16 magnitude below 2^16): 16 x 8 x 4096 x 4096 33.4 us
+// a call, 32.5 (one thread per group, four pieces always: before), 8 x 16 29.0 and 28.1.
 // Status word of this translation unit: [0] = 9 (BITDELTA_ERR_RANGE) once the split has met a magnitude of
 // 2^16 or more (it is clamped to 65504, the largest binary16 number, exactly as the GEMM kernels' own split does).
 static __device__ unsigned int g_simple_status[2];
 
 __global__ void __launch_bounds__(128) x_split_kernel(const uint16_t* __restrict__ X, uint8_t* __restrict__ X8,
-                                                      int m, int K, long long total_groups, int f16) {
+                                                      int m, int K, long long total, int f16) {
     // Let the GEMM kernel queued behind this one start its weight prefetch right away.
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (gid >= total_groups) return;
-    const int groups = K >> 5;
-    const int row = (int)(gid / groups);
-    const int g = (int)(gid - (long long)row * groups);
+    const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (id >= total) return;
+    const int quarters = K >> 3;
+    const int row = (int)(id / quarters);
+    const int k0 = (int)(id - (long long)row * quarters) >> 2 << 5, u = (int)id & 3;   // (quarters is a multiple of 4)
     const int b = row / m, t = row - b * m;
-    const uint4* src = reinterpret_cast<const uint4*>(X + (size_t)row * K + g * 32);
-    float y[32];
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(X + (size_t)row * K + k0) + u;
+    float2 y[4];   // k = 2u + 8i and the next
     bool out_of_range = false;
 #pragma unroll
-    for (int h = 0; h < 4; ++h) {
-        const uint4 v = __ldg(src + h);
-        const uint32_t q[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            y[h * 8 + 2 * i] = io16_to_float((uint16_t)(q[i] & 0xFFFFu), f16);
-            y[h * 8 + 2 * i + 1] = io16_to_float((uint16_t)(q[i] >> 16), f16);
-            if (!f16 && (((q[i] & 0x7FFFu) >= 0x4780u) || (((q[i] >> 16) & 0x7FFFu) >= 0x4780u))) out_of_range = true;
-        }
+    for (int i = 0; i < 4; ++i) {
+        const uint32_t q = __ldg(src + 4 * i);
+        y[i] = make_float2(io16_to_float((uint16_t)(q & 0xFFFFu), f16), io16_to_float((uint16_t)(q >> 16), f16));
+        if (!f16 && (((q & 0x7FFFu) >= 0x4780u) || (((q >> 16) & 0x7FFFu) >= 0x4780u))) out_of_range = true;
     }
     if (out_of_range) {
 #pragma unroll
-        for (int i = 0; i < 32; ++i) y[i] = fminf(fmaxf(y[i], -65504.f), 65504.f);
+        for (int i = 0; i < 4; ++i) y[i] = make_float2(fminf(fmaxf(y[i].x, -65504.f), 65504.f), fminf(fmaxf(y[i].y, -65504.f), 65504.f));
         atomicCAS(&g_simple_status[0], 0u, 9u);
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        uint32_t w[8];
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            uint32_t acc = 0;
+        uint32_t w0 = 0, w1 = 0;
+        if (q < 3 || f16 || out_of_range) {
+            uint32_t pc[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                const uint8_t pc = e5m2_round(y[c + 8 * i]);
-                y[c + 8 * i] -= e5m2_value(pc);
-                acc |= (uint32_t)pc << (8 * i);
+                const __nv_fp8x2_storage_t v = __nv_cvt_float2_to_fp8x2(y[i], __NV_SATFINITE, __NV_E5M2);
+                const float2 back = __half22float2(__half2(__nv_cvt_fp8x2_to_halfraw2(v, __NV_E5M2)));
+                y[i].x -= back.x;
+                y[i].y -= back.y;
+                pc[i] = v;
             }
-            w[c] = acc;
+            const uint32_t lo = __byte_perm(pc[0], pc[1], 0x5410), hi = __byte_perm(pc[2], pc[3], 0x5410);
+            w0 = __byte_perm(lo, hi, 0x6420);
+            w1 = __byte_perm(lo, hi, 0x7531);
         }
-        uint4* dst = reinterpret_cast<uint4*>(X8 + ((size_t)(b * 4 + q) * m + t) * K + g * 32);
-        dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
-        dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
+        *reinterpret_cast<uint2*>(X8 + ((size_t)(b * 4 + q) * m + t) * K + k0 + 8 * u) = make_uint2(w0, w1);
     }
 }
 
@@ -212,7 +205,7 @@ cudaError_t read_simple_status(unsigned int out[2]) {
 }
 
 cudaError_t launch_x_split(const void* X, uint8_t* X8, int B, int m, int K, int f16, cudaStream_t stream) {
-    const long long total = (long long)B * m * (K >> 5);
+    const long long total = (long long)B * m * (K >> 3);
     const int threads = 128;
     const long long blocks = (total + threads - 1) / threads;
     x_split_kernel<<<(unsigned)blocks, threads, 0, stream>>>(reinterpret_cast<const uint16_t*>(X), X8, m, K, total, f16);
