@@ -138,10 +138,13 @@ int bitdelta_workspace_init(void* workspace, size_t workspace_bytes, void* cuda_
  * is still running; it reads X and writes Y and the workspace only after that
  * kernel has completed.  W_base, bits and alpha must therefore not be produced
  * by the kernel queued directly before the call (weights are static in the
- * intended use); X may be.  The library's own producers are covered: the
- * first bitdelta_gemm call after a bitdelta_pack or bitdelta_compress call is
- * launched without the early start.  BITDELTA_EARLY_START=0 in the environment
- * turns the early start off altogether.
+ * intended use); X may be.  The library's own producers are covered: after a
+ * bitdelta_pack or bitdelta_compress call, whatever its stream, the next
+ * bitdelta_gemm call on each stream (of each device; in each capture) is launched
+ * without the early start.  Replaying a captured producer is a launch that the
+ * library does not see: like any other kernel that writes weights, it must not be
+ * what is queued directly before an eager call (within one graph it is covered).
+ * BITDELTA_EARLY_START=0 in the environment turns the early start off altogether.
  */
 int bitdelta_gemm(const void* X, const void* W_base, const uint32_t* bits, const float* alpha,
                   void* Y, int B, int m, int N, int K,

@@ -16,7 +16,7 @@ CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(CSRC, "build")
 LIB = os.path.join(HERE, "libbitdelta.so")
 SOURCES = ["api.cu", "gemm_tc.cu", "gemm_fp4.cu", "gemm_row.cu", "compress.cu", "kernels_simple.cu"]
-HEADERS = ["ptx.cuh", "plan.h", "gemm_tc.h", "gemm_common.cuh", "gemm_row.h", "row_plan.h", os.path.join("..", "..", "include", "bitdelta.h")]
+HEADERS = ["ptx.cuh", "plan.h", "gemm_tc.h", "gemm_common.cuh", "gemm_row.h", "row_plan.h", "early_start.h", os.path.join("..", "..", "include", "bitdelta.h")]
 ARCH = ["-gencode", "arch=compute_100a,code=sm_100a"]
 
 

@@ -11,6 +11,7 @@
 #include <mutex>
 
 #include "../../include/bitdelta.h"
+#include "early_start.h"
 #include "gemm_row.h"
 #include "gemm_tc.h"
 #include "plan.h"
@@ -23,9 +24,9 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[BITDELTA_NOALLO
 namespace {
 
 std::atomic<unsigned long long> g_launches{0};
-// Set by the entry points that PRODUCE what the GEMM prefetches before its grid dependency is resolved (sign words,
-// alpha: bitdelta_pack, bitdelta_compress); the next GEMM call then launches fully serialised, once.
-std::atomic<int> g_weights_just_written{0};
+// The entry points that PRODUCE what the GEMM prefetches before its grid dependency is resolved (sign words, alpha: bitdelta_pack,
+// bitdelta_compress) note it here; the next GEMM call on each stream then launches fully serialised, once.
+bd::ProducerNote g_producers;
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
@@ -183,6 +184,23 @@ bool early_start_enabled() {
     return !(e && e[0] == '0');
 }
 
+// The stream of a call, for the producers' note.  The default stream cannot be captured; the per-thread one is another in every thread.
+bool stream_key(int device, cudaStream_t stream, bd::StreamKey* key) {
+    static thread_local char this_thread;
+    key->device = device;
+    key->stream = stream == cudaStreamPerThread ? static_cast<const void*>(&this_thread) : static_cast<const void*>(stream);
+    key->capture = 0;
+    if (stream == nullptr || stream == cudaStreamLegacy) return true;
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    unsigned long long id = 0;
+    if (cudaStreamGetCaptureInfo(stream, &status, &id) != cudaSuccess || status == cudaStreamCaptureStatusInvalidated) {
+        cudaGetLastError();   // (the launch reports what is wrong with the stream)
+        return false;
+    }
+    if (status == cudaStreamCaptureStatusActive) key->capture = id;
+    return true;
+}
+
 // The row-stream decode kernel: by default where it pays (row_plan.h); BITDELTA_ROW=1: wherever it applies, =0: never.  A choice
 // of the other decode kernels (BITDELTA_FP4 and its variants, BITDELTA_CLUSTER) leaves the call to them.
 bool take_row_kernel(int B, int m, int N, int K, int sms, bool plain, int cluster) {
@@ -259,9 +277,9 @@ int bitdelta_pack(const int8_t* S, uint32_t* bits, int B, int N, int K, void* cu
     st = check_arch(&d);
     if (st != BITDELTA_OK) return st;
     const long long words = (long long)B * N * (K / 32);
+    const bd::Producing producing(g_producers);
     if (bd::launch_pack(S, bits, words, static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess)
         return BITDELTA_ERR_CUDA;
-    g_weights_just_written.store(1);
     g_launches++;
     return BITDELTA_OK;
 }
@@ -296,10 +314,10 @@ int bitdelta_compress(const void* W_fine, const void* W_base, uint32_t* bits, fl
     DeviceInfo d;
     int st = check_arch(&d);
     if (st != BITDELTA_OK) return st;
+    const bd::Producing producing(g_producers);
     if (bd::launch_compress(W_fine, W_base, bits, alpha, static_cast<double*>(workspace), B, N, K,
                             static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess)
         return BITDELTA_ERR_CUDA;
-    g_weights_just_written.store(1);
     g_launches += 2;
     return BITDELTA_OK;
 }
@@ -387,8 +405,9 @@ static int run_gemm(const void* X, const void* W_base, const uint32_t* bits, con
         ra.TB = rp.TB; ra.rows = rp.rows; ra.groups = rp.groups; ra.units = rp.units; ra.stages = rp.stages; ra.k_stages = rp.k_stages;
         ra.s_off = rp.s_off; ra.x_off = rp.x_off; ra.stage_bytes = rp.stage_bytes;
         ra.bias = bias; ra.alpha = alpha; ra.Y = Y;
-        const bool early = early_start_enabled() && g_weights_just_written.exchange(0) == 0;
-        if (bd::launch_gemm_row(rW, rX, rB, ra, rp, early, stream) != cudaSuccess) return BITDELTA_ERR_CUDA;
+        bd::ProductStart start(g_producers, early_start_enabled(), [&](bd::StreamKey* k) { return stream_key(d.device, stream, k); });
+        if (bd::launch_gemm_row(rW, rX, rB, ra, rp, start.early, stream) != cudaSuccess) return BITDELTA_ERR_CUDA;
+        start.launched();
         g_launches++;
         return BITDELTA_OK;
     }
@@ -486,11 +505,12 @@ static int run_gemm(const void* X, const void* W_base, const uint32_t* bits, con
     args.X = X; args.bits = bits;
     { static int h = -1; if (h < 0) { const char* e = getenv("BITDELTA_HOLD"); h = (e && e[0] == '0') ? 0 : 1; } args.hold_prefetch = h; }
     // (a GEMM queued right behind the library's own pack / compress must not prefetch what they are still writing)
-    const bool early = early_start_enabled() && g_weights_just_written.exchange(0) == 0;
+    bd::ProductStart start(g_producers, early_start_enabled(), [&](bd::StreamKey* k) { return stream_key(d.device, stream, k); });
     const cudaError_t le = p.fp4
-        ? bd::launch_gemm_fp4(tmW, tmBits, args, p.grid, p.smem_bytes, early, stream)
-        : bd::launch_gemm_tc(tmW, tmX, tmX8, tmBits, args, p.grid, p.smem_bytes, early, stream);
+        ? bd::launch_gemm_fp4(tmW, tmBits, args, p.grid, p.smem_bytes, start.early, stream)
+        : bd::launch_gemm_tc(tmW, tmX, tmX8, tmBits, args, p.grid, p.smem_bytes, start.early, stream);
     if (le != cudaSuccess) return BITDELTA_ERR_CUDA;
+    start.launched();
     g_launches++;
     return BITDELTA_OK;
 }
