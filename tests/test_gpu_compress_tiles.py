@@ -1,5 +1,5 @@
 """GPU tests of the compress step where its tiles of 8192 elements end: whole and partial last tiles, one word, more tiles than blocks, more
-tenants than are staged at once."""
+tenants than are staged at once, and both."""
 import numpy as np
 import pytest
 import torch
@@ -11,7 +11,7 @@ from paper_2609_36800_b200 import synth
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("shape", [(1, 1, 32), (2, 255, 32), (2, 256, 32), (3, 257, 32), (1, 2369, 1024), (2, 300, 8192 + 96), (33, 17, 512)], ids=str)
+@pytest.mark.parametrize("shape", [(1, 1, 32), (2, 255, 32), (2, 256, 32), (3, 257, 32), (1, 2369, 1024), (2, 300, 8192 + 96), (33, 17, 512), (35, 2400, 1024)], ids=str)
 def test_tile_edges(shape):
     B, N, K = shape
     fine, W = synth.make_fine_weights(B, N, K, seed=B + N + K)
