@@ -69,7 +69,9 @@ int bitdelta_unpack(const uint32_t* bits, int8_t* S, int B, int N, int K, void* 
  *             (per-block partial sums; needs no preparation, is fully rewritten).
  * The signs are exact (compared on the bf16 values); alpha is summed in double in a fixed order, so it is
  * reproducible bit for bit and within ~1e-7 relative of the exact mean.  K must be a multiple of 32;
- * W_fine, W_base and bits 16-byte aligned.  Asynchronous on the stream.
+ * W_fine, W_base and bits 16-byte aligned.  Asynchronous on the stream; a kernel-side
+ * wait that expires (sign words then stay unwritten, alpha is wrong) is reported by
+ * bitdelta_last_device_status, not here.
  */
 size_t bitdelta_compress_workspace_bytes(int B, int N, int K);
 int bitdelta_compress(const void* W_fine, const void* W_base, uint32_t* bits, float* alpha, int B, int N, int K,

@@ -143,8 +143,10 @@ __global__ void gemm_simt_kernel(const uint16_t* __restrict__ X, const uint16_t*
 // produces: byte slot 4c+i holds k = c + 8i; thread u of the four makes the slots of c = 2u and 2u + 1, from
 // pairs of neighbours.  Output rows: X8[(b*4 + q)*m + t, :] for piece q.
 // Bound by latency and, with many rows, by the conversions: eight values a thread, converted in pairs, and no fourth
-// piece where the third leaves nothing (every bfloat16 magnitude below 2^16): 16 x 8 x 4096 x 4096 33.4 us
-// a call, 32.5 (one thread per group, four pieces always: before), 8 x 16 29.0 and 28.1.
+// piece where the third leaves nothing to represent (every bfloat16 magnitude below 2^16; a remainder below 2^-17 would be
+// a signed zero).  The whole call in a graph, against one thread per group and four pieces always: 16 x 8 x 4096 x 4096
+// 33.4 -> 32.5 us, 8 x 16 28.3 -> 27.4, 16 x 6 x 4096 x 5000 39.4 -> 38.5, 16 x 8 x 4096 x 11008 76.3 -> 75.2; 32 x 4 x 4096 x 4096,
+// 24 x 8 x 11008 x 4096 and 32 x 8 x 14336 x 4096 level.
 // Status word of this translation unit: [0] = 9 (BITDELTA_ERR_RANGE) once the split has met a magnitude of
 // 2^16 or more (it is clamped to 65504, the largest binary16 number, exactly as the GEMM kernels' own split does).
 static __device__ unsigned int g_simple_status[2];

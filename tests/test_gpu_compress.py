@@ -11,12 +11,13 @@ pytestmark = pytest.mark.gpu
 # everything else in double in a fixed order; the oracle sums in double.  Worst case ~2.4e-7 relative.
 ALPHA_RTOL = 1e-6
 
+# (tiles are runs of 8192 elements of the flat matrix; its edges: test_gpu_compress_tiles.py)
 SHAPES = [
-    (1, 8, 32),          # one word per row
-    (2, 16, 1024),       # exactly one warp tile per row
-    (3, 33, 1056),       # ragged: a second, mostly empty tile per row; rows not a multiple of the block
-    (5, 130, 4096),      # several tiles per row
-    (40, 9, 2048),       # more tenants than one shared-memory chunk
+    (1, 8, 32),          # a partial tile only: eight words
+    (2, 16, 1024),       # two whole tiles, one row of 32 words after the other
+    (3, 33, 1056),       # four whole tiles and a remainder, rows that start inside a warp's run
+    (5, 130, 4096),      # 65 tiles, two rows each
+    (40, 9, 2048),       # more tenants than are staged at once
 ]
 
 

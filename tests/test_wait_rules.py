@@ -23,3 +23,13 @@ def test_waits_of_the_several_tenants_roles():
     assert re.search(r"wait_bar\(", branch[:branch.index("tmem_st32")]) and "warp_all(wait_bar(aempty_g" in branch[:branch.index("tmem_st32")]
     for wait in (r"wait_bar\(smem_u32\(&ctl->bfull\[bslot\]\), bphase, abort_flag, 6\);", r"wait_bar\(smem_u32\(&ctl->accfull\), accphase, abort_flag, 8\);"):
         assert re.search(wait + r"\s+if constexpr \(kGrouped\) ok = warp_all\(ok\);", src), wait
+
+
+def test_waits_of_the_compress_kernel():
+    # (the producer is one thread; the consumers' shuffles and their arrivals come behind a wait whose answer the warp shares)
+    src = open(os.path.join(CSRC, "compress.cu")).read()
+    body = src[src.index("compress_kernel("):src.index("__global__ void compress_finish_kernel(")]
+    producer, consumers = body[:body.index("// Lane l's 64 bytes of a tile")], body[body.index("// Lane l's 64 bytes of a tile"):]
+    assert producer.count("wait_bar(") == 1 and producer.index("if (lane == 0) {") < producer.index("wait_bar(")
+    waits = re.findall(r"[^\n]*wait_bar\([^\n]*", consumers)
+    assert len(waits) == 1 and "ok = warp_all(ok && wait_bar(" in waits[0], waits
