@@ -142,10 +142,11 @@ int bitdelta_workspace_init(void* workspace, size_t workspace_bytes, void* cuda_
  * by the kernel queued directly before the call (weights are static in the
  * intended use); X may be.  The library's own producers are covered: after a
  * bitdelta_pack or bitdelta_compress call, whatever its stream, the next
- * bitdelta_gemm call on each stream (of each device; in each capture) is launched
- * without the early start.  Replaying a captured producer is a launch that the
- * library does not see: like any other kernel that writes weights, it must not be
- * what is queued directly before an eager call (within one graph it is covered).
+ * bitdelta_gemm call on each stream of each device is launched without the early
+ * start; of the calls recorded in a capture, those behind a producer recorded in the
+ * same capture.  Replaying a captured producer is a launch that the library does not
+ * see: like any other kernel that writes weights, it must not be what is queued
+ * directly before an eager call.
  * BITDELTA_EARLY_START=0 in the environment turns the early start off altogether.
  */
 int bitdelta_gemm(const void* X, const void* W_base, const uint32_t* bits, const float* alpha,

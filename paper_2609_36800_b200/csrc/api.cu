@@ -25,7 +25,7 @@ namespace {
 
 std::atomic<unsigned long long> g_launches{0};
 // The entry points that PRODUCE what the GEMM prefetches before its grid dependency is resolved (sign words, alpha: bitdelta_pack,
-// bitdelta_compress) note it here; the next GEMM call on each stream then launches fully serialised, once.
+// bitdelta_compress) note it here; the next GEMM call on each stream (or in the same capture) then launches fully serialised, once.
 bd::ProducerNote g_producers;
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -277,7 +277,7 @@ int bitdelta_pack(const int8_t* S, uint32_t* bits, int B, int N, int K, void* cu
     st = check_arch(&d);
     if (st != BITDELTA_OK) return st;
     const long long words = (long long)B * N * (K / 32);
-    const bd::Producing producing(g_producers);
+    const bd::Producing producing(g_producers, [&](bd::StreamKey* k) { return stream_key(d.device, static_cast<cudaStream_t>(cuda_stream), k); });
     if (bd::launch_pack(S, bits, words, static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess)
         return BITDELTA_ERR_CUDA;
     g_launches++;
@@ -314,7 +314,7 @@ int bitdelta_compress(const void* W_fine, const void* W_base, uint32_t* bits, fl
     DeviceInfo d;
     int st = check_arch(&d);
     if (st != BITDELTA_OK) return st;
-    const bd::Producing producing(g_producers);
+    const bd::Producing producing(g_producers, [&](bd::StreamKey* k) { return stream_key(d.device, static_cast<cudaStream_t>(cuda_stream), k); });
     if (bd::launch_compress(W_fine, W_base, bits, alpha, static_cast<double*>(workspace), B, N, K,
                             static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess)
         return BITDELTA_ERR_CUDA;
